@@ -82,6 +82,7 @@ struct StageParams {
     const double* trig_d;  // cos, sin of the dimension-2 coordinate: [cos(0..n2-1), sin(0..n2-1)]
     const float* trig_f;
     double weno_floor[kMaxDim];   // additive floor of the WENO5 epsilon per dimension, in raw-difference units
+    double weno_floor12[kMaxDim]; // 12 times that (the FP64 smoothness sums are scaled by 12)
     double half_inv_dx[kMaxDim];  // 1 / (2 dx): raw differences to (p- + p+)/2 and (p+ - p-)/2
     double half_inv_dx6[kMaxDim]; // 1 / (12 dx): the same from six times the raw differences (WENO5)
     int alpha_global;             // dissipation alpha_d = alpha_g[d] (global LF) instead of alpha_d(x)
@@ -112,6 +113,7 @@ inline StageParams finalize(StageParams p) {
         p.half_inv_dx_f[d] = (float)p.half_inv_dx[d];
         p.alpha_g_f[d] = (float)p.alpha_g[d];
         p.weno_floor_f[d] = (float)p.weno_floor[d];
+        p.weno_floor12[d] = 12.0 * p.weno_floor[d];
     }
     for (int k = 0; k < 8; ++k) p.params_f[k] = (float)p.params[k];
     p.dt_f = (float)p.dt;
@@ -135,7 +137,8 @@ struct UpwindParams {
     const void* u;
     void* pm;
     void* pp;
-    double weno_floor;
+    double weno_floor;  // FP64: times 12 (see StageParams)
+    double inv_6dx;     // 1 / (6 dx)
 };
 
 // Launch configuration of the row-tiled stage kernel (rows_kernel.cuh).

@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(kBX * kBY) stage_kernel(const StageParams P) {
         for (int d = 0; d < D; ++d) {
             T v[7];
             gather7<T>(u, flat, idx[d], g.n[d], g.stride[d], (g.periodic_mask >> d) & 1u, g.extrap, v);
-            upwind_pair<T, SCHEME>(v, g.dx[d], g.inv_dx[d], SP<T>::floor(P, d), pm[d], pp[d]);
+            upwind_pair<T, SCHEME>(v, g.dx[d], 2.0 * P.half_inv_dx6[d], SP<T>::floor(P, d), pm[d], pp[d]);
         }
         T y = lf_term<T, D>(P, idx, pm, pp);
         if (P.brt_min0) y = fmin(y, T(0));
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kBX * kBY) upwind_kernel(const UpwindParams P)
         const int d = P.dim;
         T v[7], pm, pp;
         gather7<T>(u, flat, idx[d], g.n[d], g.stride[d], (g.periodic_mask >> d) & 1u, g.extrap, v);
-        upwind_pair<T, SCHEME>(v, g.dx[d], g.inv_dx[d], T(P.weno_floor), pm, pp);
+        upwind_pair<T, SCHEME>(v, g.dx[d], P.inv_6dx, T(P.weno_floor), pm, pp);
         static_cast<T*>(P.pm)[flat] = pm;
         static_cast<T*>(P.pp)[flat] = pp;
     }

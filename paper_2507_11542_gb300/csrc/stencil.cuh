@@ -5,10 +5,12 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 #include "../../include/hj.h"
 #include "hj_internal.h"
+#include "weno_iface.cuh"
 
 namespace hj {
 
@@ -21,9 +23,10 @@ __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, 
 
 // |x|, and the maximum of two non-negative values, for FP64 as integer
 // operations on the bit patterns (non-negative doubles order like their bits):
-// exact, and off the FP64 pipe that bounds the FP64 kernels. FP32 as usual.
+// exact, and off the FP64 pipe that bounds the FP64 kernels (|x| on the high
+// word alone: a 64-bit mask is compiled to an FP64 addition). FP32 as usual.
 __device__ __forceinline__ double absv(double a) {
-    return __longlong_as_double(__double_as_longlong(a) & 0x7fffffffffffffffLL);
+    return __hiloint2double(__double2hiint(a) & 0x7fffffff, __double2loint(a));
 }
 __device__ __forceinline__ float absv(float a) { return fabsf(a); }
 __device__ __forceinline__ double max_nonneg(double a, double b) {
@@ -80,25 +83,10 @@ __device__ __forceinline__ void gather7(const T* __restrict__ u, long long idx, 
 // weights are homogeneous of degree zero in the differences, so working on
 // raw differences and dividing by dx once at the end is the same scheme when
 // the epsilon floor is scaled by dx^2 (weno_floor).
-// The two sides share the second differences of windows (r1,r2,r3) and
-// (r2,r3,r4) and two of their candidate stencils.
+// FP64 evaluates the two interfaces of the node (weno_iface). In FP32 the two
+// sides share the second differences of windows (r1,r2,r3) and (r2,r3,r4) and
+// two of their candidate stencils.
 // ---------------------------------------------------------------------------
-// FP64: weights c_k/(S_k+eps)^2 normalised with one division,
-//   p = sum_k c_k q_k prod_{j!=k} d_j / sum_k c_k prod_{j!=k} d_j,  d_k = (S_k+eps)^2.
-// On exactly flat data every d_k underflows and every q_k is zero: return q2.
-__device__ __forceinline__ double weno_combine(double q1, double q2, double q3, double s1, double s2, double s3,
-                                               double eps, double scale) {
-    const double d1 = (s1 + eps) * (s1 + eps);
-    const double d2 = (s2 + eps) * (s2 + eps);
-    const double d3 = (s3 + eps) * (s3 + eps);
-    const double w1 = 0.1 * (d2 * d3);
-    const double w2 = 0.6 * (d1 * d3);
-    const double w3 = 0.3 * (d1 * d2);
-    const double num = w1 * q1 + w2 * q2 + w3 * q3;
-    const double den = w1 + w2 + w3;
-    return (den > 0.0) ? num / (den * scale) : q2 / scale;
-}
-
 // FP32: the epsilon floor keeps (S+eps)^2 >= 1e-36 (normal), so the direct
 // form with fast reciprocals cannot overflow or divide by zero.
 __device__ __forceinline__ float weno_combine(float q1, float q2, float q3, float s1, float s2, float s3,
@@ -110,8 +98,17 @@ __device__ __forceinline__ float weno_combine(float q1, float q2, float q3, floa
     return num * __fdividef(1.0f, (a1 + a2 + a3) * scale);
 }
 
-template <typename T>
-__device__ __forceinline__ void weno5_pair(const T v[7], T dx, T floor_raw, T& pm, T& pp) {
+__device__ __forceinline__ void weno5_pair(const double v[7], double inv_6dx, double floor12, double& pm, double& pp) {
+    const double r1 = v[2] - v[1], r2 = v[3] - v[2], r3 = v[4] - v[3], r4 = v[5] - v[4];
+    double unused, pm6, pp6;
+    weno_iface(v[1] - v[0], r1, r2, r3, r4, floor12, unused, pm6);
+    weno_iface(r1, r2, r3, r4, v[6] - v[5], floor12, pp6, unused);
+    pm = pm6 * inv_6dx;
+    pp = pp6 * inv_6dx;
+}
+
+__device__ __forceinline__ void weno5_pair(const float v[7], float dx, float floor_raw, float& pm, float& pp) {
+    using T = float;
     const T r0 = v[1] - v[0], r1 = v[2] - v[1], r2 = v[3] - v[2];
     const T r3 = v[4] - v[3], r4 = v[5] - v[4], r5 = v[6] - v[5];
     const T c13 = T(13) / T(12);
@@ -200,9 +197,10 @@ __device__ __forceinline__ void eno_pair(const T v[7], T dx, int order, T& pm, T
 }
 
 template <typename T, int SCHEME>
-__device__ __forceinline__ void upwind_pair(const T v[7], double dx, double inv_dx, T floor_raw, T& pm, T& pp) {
+__device__ __forceinline__ void upwind_pair(const T v[7], double dx, double inv_6dx, T floor, T& pm, T& pp) {
     if constexpr (SCHEME == HJ_WENO5) {
-        weno5_pair<T>(v, T(dx), floor_raw, pm, pp);
+        if constexpr (std::is_same<T, double>::value) weno5_pair(v, inv_6dx, floor, pm, pp);
+        else weno5_pair(v, T(dx), floor, pm, pp);
     } else {
         eno_pair<T>(v, T(dx), SCHEME, pm, pp);
     }
@@ -228,7 +226,8 @@ template <> struct SP<double> {
     static __device__ __forceinline__ double dt(const StageParams& P) { return P.dt; }
     static __device__ __forceinline__ double cv(const StageParams& P) { return P.cv; }
     static __device__ __forceinline__ double cu(const StageParams& P) { return P.cu; }
-    static __device__ __forceinline__ double floor(const StageParams& P, int d) { return P.weno_floor[d]; }
+    // 12 times the floor (the scale of the FP64 smoothness sums)
+    static __device__ __forceinline__ double floor(const StageParams& P, int d) { return P.weno_floor12[d]; }
 };
 template <> struct SP<float> {
     static __device__ __forceinline__ float lo(const StageParams& P, int d) { return P.lo_f[d]; }

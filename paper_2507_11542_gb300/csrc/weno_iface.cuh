@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "../../include/hj.h"
+#include "weno_weights64.cuh"
 
 namespace hj {
 
@@ -39,9 +40,9 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return r;
 }
 
-// FP32, in the rescaled form of the FP64 interface below (smoothness values
-// and epsilon times 4, ideal weights times 10, results times 6; the caller
-// divides the 6 out with 1/(2 dx)), with one reciprocal per weight and per
+// FP32, rescaled in ways that leave every weight unchanged: smoothness values
+// and epsilon times 4 (S' = 13/3 t^2 + u^2), ideal weights times 10; results
+// times 6 (the caller divides the 6 out with 1/(2 dx)); with one reciprocal per weight and per
 // side: (S' + eps')^2 >= (4e-18)^2 stays a normal number, so the approximate
 // reciprocals neither overflow nor divide by zero. No a*b + c is left for the
 // compiler to contract, so every inlined copy rounds alike.
@@ -75,19 +76,10 @@ __device__ __forceinline__ void weno_iface(float e1, float e2, float e3, float e
     pp_j = fmaf(-numR, rcp_approx(DR), psi6);
 }
 
-// Integer maximum of non-negative doubles (their bit patterns order alike):
-// keeps the epsilon's max off the FP64 pipe.
-__device__ __forceinline__ double nonneg_max(double a, double b) {
-    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
-    return __longlong_as_double(ia > ib ? ia : ib);
-}
-
-__device__ __forceinline__ double abs_bits(double a) {
-    return __longlong_as_double(__double_as_longlong(a) & 0x7fffffffffffffffLL);
-}
-
 // 1/x for a positive normal double: the hardware estimate refined by two
 // Newton-Raphson steps r <- r + r (1 - x r) (each squares the relative error).
+// The interface no longer needs it (its reciprocals are integer); it stays as
+// the library's FP64 reciprocal, held against 1/x by its test.
 __device__ __forceinline__ double rcp_newton(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -97,75 +89,52 @@ __device__ __forceinline__ double rcp_newton(double x) {
     return fma(r, e, r);
 }
 
-// FP64. Weights normalised by products of the d_k = (S'_k + eps')^2:
-//   w_k = c_k prod_{i!=k} d_i / sum_m c_m prod_{i!=m} d_i,
-// and both sides share one reciprocal 1/(DL DR). Three rescalings that leave
-// every weight unchanged save FP64 operations (the FP64 pipe bounds this
-// kernel):
-//   * the smoothness indicators and epsilon times 4: S' = 13/3 t^2 + u^2,
-//     eps' = 4e-6 max(e_k^2) + 4 floor;
-//   * the ideal weights times 10: DL = PA + 6 PB + 3 PC, DR = 3 PA + 6 PB + PC;
-//   * both results times 6: 6 p- = (-e2 + 5e3 + 2e4) + (2X + 3Y)/DL and
-//     6 p+ = 6 phi2 + 3 (e2 - e4) - (3X + 2Y)/DR, X = PA T1, Y = PC T2
-//     (2X + 3Y = 2(X+Y) + Y, 3X + 2Y = 2(X+Y) + X).
-// The caller divides the factor 6 out with its 1/(2 dx) (iface_times6).
-// The core takes what consecutive interfaces along a line share (Weno5Line):
-// tA, tB, tC (the second differences of the windows' first differences), q =
-// 13/3 t^2 for each, the differences d23 = e3 - e2 and d34 = e4 - e3 of the
-// first differences, and the third differences T1 = tA - tB, T2 = tB - tC.
+// FP64. The first, second and third differences and the two results are FP64,
+// the weights 64-bit integer arithmetic (weno_weights64.cuh, which takes the
+// smoothness sums times 12 and the ideal weights times 10: both leave every
+// weight unchanged). Both results are times 6, written around the interface's
+// own difference so that one rounding alone happens at their magnitude:
+//   6 p- = 6 e3 + (2 d34 + d23 + l1 T1 + l3 T2)
+//   6 p+ = 6 e3 - (2 d23 + d34 + r1 T1 + r3 T2)
+// with d23 = e3 - e2, d34 = e4 - e3 and the weights l1 = 2 w1, l3 = w3 (left),
+// r1 = w3', r3 = 2 w1' (right). The caller divides the 6 out with its
+// 1/(2 dx) (iface_times6). A non-finite difference reaches both results
+// through T1 or T2, since the weights are finite whatever their input.
+//
+// The FP64 pipe bounds this (16-20 cycles a warp instruction and SM): 25 FP64
+// instructions from five first differences, 15 along a line (Weno5Line), where
+// the weights in FP64 took 64 and 50 (1272 and 1009 cycles, now 540 and 340).
+// The core takes what consecutive interfaces along a line share: tA, tB, tC
+// (the second differences of the windows' first differences), d23, d34 and the
+// third differences T1 = tA - tB, T2 = tB - tC. floor12: 12 times the epsilon
+// floor. No a*b + c is left for the compiler to contract, so every inlined
+// copy rounds alike and results do not depend on which thread role evaluates
+// an interface.
 __device__ __forceinline__ void weno_core(double e1, double e2, double e3, double e4, double e5, double tA, double tB,
-                                          double tC, double qA, double qB, double qC, double d23, double d34,
-                                          double T1, double T2, double floor_raw, double& pp_j, double& pm_j1) {
+                                          double tC, double d23, double d34, double T1, double T2, double floor12,
+                                          double& pp_j, double& pm_j1) {
     const double uA = fma(2.0, d23, tA);   // e1 - 4e2 + 3e3
     const double uB = e2 - e4;
     const double uC = fma(-2.0, d34, tC);  // 3e3 - 4e4 + e5
-    const double SA = fma(uA, uA, qA);
-    const double SB = fma(uB, uB, qB);
-    const double SC = fma(uC, uC, qC);
-    const double amax = nonneg_max(nonneg_max(nonneg_max(abs_bits(e1), abs_bits(e2)),
-                                              nonneg_max(abs_bits(e3), abs_bits(e4))), abs_bits(e5));
-    const double eps = fma(4e-6, amax * amax, 4.0 * floor_raw);
-    // sA, sB, sC scaled by the power of two that brings the largest into
-    // [1, 2): an exact integer subtraction on the bit patterns of these
-    // positive normal numbers. eps bounds their ratios (s_min >= 3e-8 s_max:
-    // S' <= 133.4 max(e_k^2)), so DL and DR stay within [9e-16, 160] and one
-    // shared reciprocal serves every window, flat and tiny ones included.
-    // The weights do not change.
-    const long long bA = __double_as_longlong(SA + eps), bB = __double_as_longlong(SB + eps),
-                    bC = __double_as_longlong(SC + eps);
-    const long long bm = bA > bB ? (bA > bC ? bA : bC) : (bB > bC ? bB : bC);
-    const long long shift = (bm & 0x7ff0000000000000LL) - 0x3ff0000000000000LL;
-    const double sA = __longlong_as_double(bA - shift), sB = __longlong_as_double(bB - shift),
-                 sC = __longlong_as_double(bC - shift);
-    const double dA = sA * sA, dB = sB * sB, dC = sC * sC;
-    const double PA = dB * dC, PB = dA * dC, PC = dA * dB;
-    const double X = PA * T1, Y = PC * T2;
-    // no a*b + c is left for the compiler to contract: every inlined copy of
-    // this function rounds alike, so results do not depend on which thread
-    // role evaluates an interface
-    const double XY = __dadd_rn(X, Y);
-    const double numL = fma(2.0, XY, Y);  // 2X + 3Y
-    const double numR = fma(2.0, XY, X);  // 3X + 2Y
-    const double DL = fma(3.0, PC, fma(6.0, PB, PA));
-    const double DR = fma(3.0, PA, fma(6.0, PB, PC));
-    const double phi6 = fma(5.0, e3, fma(2.0, e4, -e2));  // 6 phi2
-    const double psi6 = fma(3.0, uB, phi6);               // 6 psi2
-    const double r = rcp_newton(DL * DR);
-    pm_j1 = fma(numL * DR, r, phi6);
-    pp_j = fma(-numR * DL, r, psi6);
+    const w64::u64 amax = w64::umax(w64::umax(w64::umax(w64::abs_bits(e1), w64::abs_bits(e2)),
+                                              w64::umax(w64::abs_bits(e3), w64::abs_bits(e4))), w64::abs_bits(e5));
+    const w64::Sum eps = w64::eps_sum(amax, w64::floor_term(floor12));
+    double l1, l3, r1, r3;
+    w64::weights(w64::smooth_sum(tA, uA, eps), w64::smooth_sum(tB, uB, eps), w64::smooth_sum(tC, uC, eps), l1, l3, r1,
+                 r3);
+    const double sL = fma(l3, T2, fma(l1, T1, fma(2.0, d34, d23)));
+    const double sR = fma(r3, T2, fma(r1, T1, fma(2.0, d23, d34)));
+    pm_j1 = fma(6.0, e3, sL);
+    pp_j = fma(6.0, e3, -sR);
 }
-
-// 13/3 t^2, the share of t in the rescaled smoothness indicator
-__device__ __forceinline__ double curv_sq(double t) { return (13.0 / 3.0 * t) * t; }
 
 // Six times the FP64 one-sided derivatives (weno_core), from the five first
 // differences: t as differences of the d = e_{k+1} - e_k.
-__device__ __forceinline__ void weno_iface(double e1, double e2, double e3, double e4, double e5, double floor_raw,
+__device__ __forceinline__ void weno_iface(double e1, double e2, double e3, double e4, double e5, double floor12,
                                            double& pp_j, double& pm_j1) {
     const double d12 = e2 - e1, d23 = e3 - e2, d34 = e4 - e3, d45 = e5 - e4;
     const double tA = d23 - d12, tB = d34 - d23, tC = d45 - d34;
-    weno_core(e1, e2, e3, e4, e5, tA, tB, tC, curv_sq(tA), curv_sq(tB), curv_sq(tC), d23, d34, tA - tB, tB - tC,
-              floor_raw, pp_j, pm_j1);
+    weno_core(e1, e2, e3, e4, e5, tA, tB, tC, d23, d34, tA - tB, tB - tC, floor12, pp_j, pm_j1);
 }
 
 // Whether an interface evaluation returns six times the derivatives (WENO5,
@@ -178,15 +147,14 @@ __host__ __device__ constexpr bool iface_times6() {
 
 // FP64 WENO5 along a grid line, one interface after the other: the interface
 // between nodes j and j+1 reuses four of the five first differences, two of
-// the three differences d, two of the three values tA, tB, tC and their
-// squares, and one of the two third differences of the interface before it,
-// so each step computes one of each. The results are those of weno_iface,
-// bit for bit (the same operations on the same operands).
+// the three differences d, two of the three values tA, tB, tC and one of the
+// two third differences of the interface before it, so each step computes one
+// of each. The results are those of weno_iface, bit for bit (the same
+// operations on the same operands).
 struct Weno5Line {
     double e[5];   // first differences of the current window
     double d[3];   // d23, d34, d45: differences of consecutive e
     double t[3];   // tA, tB, tC
-    double sq[3];  // 13/3 of their squares
     double T[2];   // T1, T2
     // the window of the values v0..v5 at nodes j-2 .. j+3
     __device__ __forceinline__ void start(double v0, double v1, double v2, double v3, double v4, double v5) {
@@ -194,7 +162,6 @@ struct Weno5Line {
         const double d12 = e[1] - e[0];
         d[0] = e[2] - e[1]; d[1] = e[3] - e[2]; d[2] = e[4] - e[3];
         t[0] = d[0] - d12; t[1] = d[1] - d[0]; t[2] = d[2] - d[1];
-        sq[0] = curv_sq(t[0]); sq[1] = curv_sq(t[1]); sq[2] = curv_sq(t[2]);
         T[0] = t[0] - t[1]; T[1] = t[1] - t[2];
     }
     // slide by one node: v4, v5 are the values at the new window's last two nodes
@@ -202,12 +169,10 @@ struct Weno5Line {
         e[0] = e[1]; e[1] = e[2]; e[2] = e[3]; e[3] = e[4]; e[4] = v5 - v4;
         d[0] = d[1]; d[1] = d[2]; d[2] = e[4] - e[3];
         t[0] = t[1]; t[1] = t[2]; t[2] = d[2] - d[1];
-        sq[0] = sq[1]; sq[1] = sq[2]; sq[2] = curv_sq(t[2]);
         T[0] = T[1]; T[1] = t[1] - t[2];
     }
-    __device__ __forceinline__ void eval(double floor_raw, double& pp_j, double& pm_j1) const {
-        weno_core(e[0], e[1], e[2], e[3], e[4], t[0], t[1], t[2], sq[0], sq[1], sq[2], d[0], d[1], T[0], T[1],
-                  floor_raw, pp_j, pm_j1);
+    __device__ __forceinline__ void eval(double floor12, double& pp_j, double& pm_j1) const {
+        weno_core(e[0], e[1], e[2], e[3], e[4], t[0], t[1], t[2], d[0], d[1], T[0], T[1], floor12, pp_j, pm_j1);
     }
 };
 
@@ -220,9 +185,9 @@ struct Weno5Line {
 //   e = v2 - v1, dL = e - (v1 - v0), dR = (v3 - v2) - e,
 //   c = |dL| <= |dR| ? dL : dR,  p+_j = e - c/2,  p-_{j+1} = e + c/2.
 // |a| <= |b|: for FP64 on the bit patterns (an integer comparison, exact for
-// finite values).
+// finite values; the sign is masked in the high word, see w64::abs_bits).
 __device__ __forceinline__ bool abs_le(double a, double b) {
-    return (__double_as_longlong(a) & 0x7fffffffffffffffLL) <= (__double_as_longlong(b) & 0x7fffffffffffffffLL);
+    return w64::abs_bits(a) <= w64::abs_bits(b);
 }
 __device__ __forceinline__ bool abs_le(float a, float b) { return fabsf(a) <= fabsf(b); }
 
