@@ -68,6 +68,8 @@ __device__ double node_bound(const GridDev& g, int dyn, const double* q, const d
 
 struct BoundArgs {
     GridDev g;
+    int count[kMaxDim];  // indices visited along each dimension: all of an angle's, the two ends of any other
+    long long total;     // their product
     int dyn;
     int per_dim;  // 0: max over nodes of the sum (one word); 1: max over nodes of each alpha_d (ndim words)
     double q[8];
@@ -85,13 +87,25 @@ __device__ __forceinline__ double block_max(double v, double* scratch) {
     return b;
 }
 
+// The maximum over the grid, from the nodes where it can lie. Every alpha_d
+// grows with |x_k| of the dimensions k it reads other than the heading angle:
+// it is built of products and sums of non-negative terms, and rounding keeps
+// their order, so that the rounded value grows too. |x_k| is largest at an end
+// of the dimension (rounded coordinates do not decrease along it). So the two
+// ends of each dimension and every node of the angle give the maximum over all
+// nodes, bit for bit: 404 nodes instead of 1.03 M on 101^3 (106 us for the
+// pass over every node with its FP64 divisions, now one launch of a few us).
 __global__ void __launch_bounds__(256) step_bound_kernel(const BoundArgs A) {
     double best[4] = {0.0, 0.0, 0.0, 0.0};
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long flat = (long long)blockIdx.x * blockDim.x + threadIdx.x; flat < A.g.total; flat += stride) {
+    for (long long flat = (long long)blockIdx.x * blockDim.x + threadIdx.x; flat < A.total; flat += stride) {
         int idx[4] = {0, 0, 0, 0};
         long long r = flat;
-        for (int d = 0; d < A.g.ndim; ++d) { idx[d] = (int)(r % A.g.n[d]); r /= A.g.n[d]; }
+        for (int d = 0; d < A.g.ndim; ++d) {
+            const int k = (int)(r % A.count[d]);
+            r /= A.count[d];
+            idx[d] = A.count[d] == A.g.n[d] ? k : k * (A.g.n[d] - 1);
+        }
         if (A.per_dim) {
             double a[4];
             node_alpha(A.g, A.dyn, A.q, A.trig, idx, a);
@@ -132,7 +146,13 @@ cudaError_t launch_step_bound(const GridDev& g, int dynamics, const double* para
     for (int k = 0; k < 8; ++k) A.q[k] = params[k];
     A.trig = trig_d;
     A.acc = acc;
-    long long blocks = (g.total + 255) / 256;
+    const bool angle = dynamics == HJ_DYN_AIR3D || dynamics == HJ_DYN_DUBINS4D || dynamics == HJ_DYN_ROCKETS;
+    A.total = 1;
+    for (int d = 0; d < kMaxDim; ++d) {
+        A.count[d] = d >= g.ndim ? 1 : (angle && d == 2) || g.n[d] < 2 ? g.n[d] : 2;
+        A.total *= A.count[d];
+    }
+    long long blocks = (A.total + 255) / 256;
     const long long cap = 16LL * device_sms();  // a few waves of resident blocks
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
