@@ -133,14 +133,13 @@ typedef struct hj_method {
     int32_t kernel;    /* HJ_KERNEL_AUTO (0), HJ_KERNEL_ROWS or HJ_KERNEL_NODE */
     /* Launch shape of the row kernel {ty, tz, occ, flags}, all 0 (the
      * default): picked by the context's tuner (timed once per grid, dtype,
-     * dynamics and scheme, then cached). Otherwise: ty node rows per block,
-     * tz planes per chunk along the last dimension (3-D and 4-D grids), occ 1
-     * or 2 resident blocks per SM (2: FP32 blocks of at most 544 threads);
-     * flags bit 0: blocks of n0*ty threads whose last node row also takes the
-     * row ends; bit 1: tiles away from the grid's edges keep the general body
-     * (the ENO schemes otherwise run them on a body compiled without ghost
-     * logic). Results do not depend on the shape (bit for bit). A shape that
-     * does not fit the grid is HJ_EINVAL. Used by hj_term, hj_rk3_step,
+     * dynamics and scheme, then cached). Otherwise: ty node rows per block (at
+     * most 8 are used), tz planes per chunk along the last dimension (3-D and
+     * 4-D grids); occ 1 or 2 (2: FP32 blocks of at most 544 nodes) and flags
+     * (bits 0 and 1) are checked but no longer change the launch. Results do
+     * not depend on the shape (bit for bit). A shape that does not fit the
+     * grid is HJ_EINVAL: n0 + 1 nodes (n0 with flags bit 0) by ty rows may be
+     * at most 1024 in FP32, 512 in FP64. Used by hj_term, hj_rk3_step,
      * hj_rk3_stage and hj_solve; a problem that sets it (or kernel = NODE) is
      * solved on its own by hj_solve_batch and refused by hj_server_submit. */
     int32_t tile_override[4];

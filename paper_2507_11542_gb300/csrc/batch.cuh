@@ -16,9 +16,10 @@ template <> __device__ __forceinline__ float batch_dt<float>(const BatchInst& I)
 
 // KIND: kKindFirst for stage 1, kKindCombine for stages 2 and 3.
 template <typename T, int D, int DYN, int SCHEME, int KIND>
-__global__ void __launch_bounds__(RowsLimits<T>::kMaxThreads)
-    batch_kernel(const BatchTile* __restrict__ tiles, const BatchInst* __restrict__ insts, const int stage) {
+__global__ void __launch_bounds__(RowsLimits<T>::kThreads, 1)
+    batch_kernel(const BatchTile* tiles, const BatchInst* insts, const int stage) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_wait();  // the descriptors change from step to step
     const BatchTile t = tiles[blockIdx.x];
     const BatchInst& I = insts[t.inst];
     if (I.k >= I.steps_total) return;  // this instance has finished (block-uniform)
@@ -48,7 +49,7 @@ __global__ void __launch_bounds__(RowsLimits<T>::kMaxThreads)
         R.cu = T(2.0 / 3.0);
         R.minv = I.brt == HJ_BRT_MINV;
     }
-    rows_tile<T, D, DYN, SCHEME, KIND>(I.P, R, I.ty, (int)blockDim.x, I.tz, t.row_tile, t.i2, t.chunk,
+    rows_tile<T, D, DYN, SCHEME, KIND>(I.P, R, I.sx, I.ty, (int)blockDim.x, I.tz, t.tile, t.i2, t.chunk,
                                        (int)threadIdx.x, reinterpret_cast<T*>(smem_raw));
 }
 
@@ -58,8 +59,8 @@ cudaError_t launch_batch_kind(const BatchTile* tiles, int ntiles, const BatchIns
     static std::atomic<unsigned long long> done{0};
     cudaError_t e = smem_optin(batch_kernel<T, D, DYN, SCHEME, KIND>, done);
     if (e != cudaSuccess) return e;
-    batch_kernel<T, D, DYN, SCHEME, KIND><<<ntiles, threads, smem, s>>>(tiles, insts, stage);
-    return cudaGetLastError();
+    return launch_dependent(batch_kernel<T, D, DYN, SCHEME, KIND>, dim3(ntiles), dim3(threads), smem, s, tiles, insts,
+                            stage);
 }
 
 template <typename T, int D, int DYN, int SCHEME>

@@ -23,6 +23,7 @@ cudaError_t launch_batch_stage_f32(const BatchTile* tiles, int ntiles, const Bat
 // tested first: other lanes' descriptors may be advancing concurrently).
 __global__ void batch_advance_kernel(BatchInst* insts, int n, int lane_lo, int lane_hi) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_wait();
     if (i >= n) return;
     BatchInst& I = insts[i];
     if (I.lane < lane_lo || I.lane > lane_hi) return;
@@ -42,8 +43,7 @@ __global__ void batch_advance_kernel(BatchInst* insts, int n, int lane_lo, int l
 }
 
 cudaError_t launch_batch_advance(BatchInst* insts, int n, int lane_lo, int lane_hi, cudaStream_t s) {
-    batch_advance_kernel<<<(n + 127) / 128, 128, 0, s>>>(insts, n, lane_lo, lane_hi);
-    return cudaGetLastError();
+    return launch_dependent(batch_advance_kernel, dim3((n + 127) / 128), dim3(128), 0, s, insts, n, lane_lo, lane_hi);
 }
 
 }  // namespace hj

@@ -127,7 +127,7 @@ bool Engine::eligible(const hj_problem* p) {
     const GridDev G = make_grid(&p->grid, p->method.extrap);
     const bool rk3_node = (p->method.order == 0 || p->method.order == 3) && p->method.alpha_mode == HJ_ALPHA_NODE;
     return rk3_node && default_launch(&p->method) && rows_eligible(G, p->method.scheme, p->method.dynamics, p->dtype) &&
-           G.n[0] + 1 <= max_block_threads(p->dtype);
+           G.n[0] + 1 <= rows_max_nodes(p->dtype == HJ_F64);
 }
 
 // The arena layout of one instance, as offsets from the start of its block:
@@ -361,10 +361,11 @@ hj_status Engine::activate(std::vector<int>* failed) {
         // members already stepping keep their device state; only their tile shape is refreshed
         for (int m : members)
             if (std::find(fresh.begin(), fresh.end(), m) == fresh.end())
-                HJ_CUDA(ctx_, cudaMemcpyAsync(reinterpret_cast<char*>(d_insts_ + m) + offsetof(BatchInst, ty),
-                                              &h_insts_[m].ty, 2 * sizeof(int), cudaMemcpyHostToDevice, stream_));
+                HJ_CUDA(ctx_, cudaMemcpyAsync(reinterpret_cast<char*>(d_insts_ + m) + offsetof(BatchInst, sx),
+                                              &h_insts_[m].sx, 3 * sizeof(int), cudaMemcpyHostToDevice, stream_));
     }
     for (int si : ok) {
+        h_insts_[si].sx = slots[si].sx;
         h_insts_[si].ty = slots[si].ty;
         h_insts_[si].tz = slots[si].tz;
         HJ_CUDA(ctx_, cudaMemcpyAsync(d_insts_ + si, &h_insts_[si], sizeof(BatchInst), cudaMemcpyHostToDevice, stream_));
@@ -377,24 +378,27 @@ hj_status Engine::activate(std::vector<int>* failed) {
 }
 
 namespace {
-void tile_shape(const Slot& S, int threads, int tz_target, int* ty, int* tz) {
-    const int nx = S.G.n[0], ny = S.G.n[1];
-    // node rows: the most whose block (rows_block_threads) fits `threads`
-    int t = 1;
-    while (t < ny && rows_block_threads(nx, t + 1, threads) <= threads) ++t;
-    while (t > 1 && rows_smem(nx, t, S.es) > 200 * 1024) --t;
-    *ty = t;
+void tile_shape(const Slot& S, int threads, int tz_target, int* sx, int* ty, int* tz) {
+    // the most rows, and the widest segment of them whose node and edge threads fit the block
+    *ty = std::min(kRowsMaxTy, S.G.n[1]);
+    int nn = threads - 32;
+    do {
+        *sx = rows_segment(S.G.n[0], *ty, nn);
+        nn -= 32;
+    } while (rows_node_threads(*sx, *ty) + rows_edge_threads(*sx) > threads);
     const int D = S.G.ndim;
     *tz = D >= 3 ? std::max(1, std::min(tz_target, S.G.n[D - 1])) : 1;
 }
+int plane_tiles(const Slot& S) {
+    return ((S.G.n[0] + S.sx - 1) / S.sx) * ((S.G.n[1] + S.ty - 1) / S.ty);
+}
 long long tiles_of(const Slot& S) {
     const int D = S.G.ndim;
-    return (long long)((S.G.n[1] + S.ty - 1) / S.ty) * (D >= 3 ? (S.G.n[D - 1] + S.tz - 1) / S.tz : 1) *
-           (D == 4 ? S.G.n[2] : 1);
+    return (long long)plane_tiles(S) * (D >= 3 ? (S.G.n[D - 1] + S.tz - 1) / S.tz : 1) * (D == 4 ? S.G.n[2] : 1);
 }
 void append_tiles(const Slot& S, int si, std::vector<BatchTile>* out) {
     const int D = S.G.ndim;
-    const int rt = (S.G.n[1] + S.ty - 1) / S.ty;
+    const int rt = plane_tiles(S);
     const int ns = D >= 3 ? S.G.n[D - 1] : 1;
     const int nch = D >= 3 ? (ns + S.tz - 1) / S.tz : 1;
     const int n2 = D == 4 ? S.G.n[2] : 1;
@@ -407,30 +411,31 @@ void append_tiles(const Slot& S, int si, std::vector<BatchTile>* out) {
 // The group's block size and planes per tile: measured once per (dtype,
 // dimension, dynamics, scheme) and context on the members at hand, then reused.
 hj_status Engine::shape_group(Group& g, const std::vector<int>& members, const std::vector<int>& fresh) {
-    int max_nx = 0;
-    for (int m : members) max_nx = std::max(max_nx, slots[m].G.n[0]);
     auto apply = [&](int threads, int tzt) {
         g.threads = threads;
         g.tz_target = tzt;
         g.smem = 0;
         for (int m : members) {
-            tile_shape(slots[m], threads, tzt, &slots[m].ty, &slots[m].tz);
-            g.smem = std::max(g.smem, rows_smem(slots[m].G.n[0], slots[m].ty, slots[m].es));
+            tile_shape(slots[m], threads, tzt, &slots[m].sx, &slots[m].ty, &slots[m].tz);
+            g.smem = std::max(g.smem, rows_smem(slots[m].sx, slots[m].es));
+            h_insts_[m].sx = slots[m].sx;
             h_insts_[m].ty = slots[m].ty;
             h_insts_[m].tz = slots[m].tz;
         }
     };
     const std::vector<long long> key = {g.dtype, g.ndim, g.dyn, g.scheme};
     auto it = ctx_->batch_shape.find(key);
-    if (it != ctx_->batch_shape.end() && it->second.first >= max_nx + 1) {
+    if (it != ctx_->batch_shape.end()) {
         apply(it->second.first, it->second.second);
         return HJ_OK;
     }
     std::vector<std::pair<int, int>> cands;
-    for (int threads : {256, 512, 1024})
-        if (threads <= max_block_threads(g.dtype) && threads >= max_nx + 1)
-            for (int tzt : {4, 8, 16, 32}) cands.push_back({threads, tzt});
-    if (cands.empty()) cands.push_back({std::min(((max_nx + 1 + 31) / 32) * 32, max_block_threads(g.dtype)), 8});
+    for (int threads : {128, 192, 256, 320, 448, 576})
+        if (threads <= max_block_threads(g.dtype)) {
+            if (g.ndim < 3) cands.push_back({threads, 1});
+            else
+                for (int tzt : {4, 8, 16, 32}) cands.push_back({threads, tzt});
+        }
     std::pair<int, int> best = cands[0];
     if (cands.size() > 1) {
         cudaEvent_t e0, e1;
@@ -519,7 +524,7 @@ hj_status Engine::rebuild_tiles() {
             append_tiles(slots[i], i, &g.tiles);
             // tiles of lanes above this instance's start after it
             for (int l = slots[i].lane + 1; l < kLanes; ++l) g.lane_off[l] = g.tiles.size();
-            g.smem = std::max(g.smem, rows_smem(slots[i].G.n[0], slots[i].ty, slots[i].es));
+            g.smem = std::max(g.smem, rows_smem(slots[i].sx, slots[i].es));
         }
         tiles_total_ += (long long)g.tiles.size();
         if (g.tiles.empty()) continue;

@@ -47,7 +47,7 @@ struct Slot {
     bool angles = false;
     int group = -1;
     int lane = 0;                    // rate class (Engine::init with lanes)
-    int ty = 1, tz = 1;
+    int sx = 1, ty = 1, tz = 1;
     Schedule S;
     double sbi = 0.0;
     long long steps_total = 0, k_host = 0;

@@ -308,23 +308,10 @@ bool rows_eligible(const GridDev& G, int scheme, int dynamics, int dtype, int ke
         return false;
     for (int d = 0; d < G.ndim; ++d)
         if (G.n[d] < 4) return false;
-    if (G.n[0] + 1 > rows_max_threads(dtype == HJ_F64)) return false;
+    if (G.n[0] + 1 > rows_max_nodes(dtype == HJ_F64)) return false;
     if (G.ndim == 4 && G.n[2] > 65535) return false;
     if (G.total >= (1LL << 31)) return false;  // the row kernel indexes with 32-bit integers
     return true;
-}
-
-RowsCfg make_rows_cfg(const GridDev& G, int ty, int tz, int dtype) {
-    RowsCfg c;
-    c.ty = ty;
-    c.nt = rows_block_threads(G.n[0], ty, rows_max_threads(dtype == HJ_F64));
-    c.occ = 1;
-    c.split = 0;
-    c.row_tiles = (G.n[1] + ty - 1) / ty;
-    const int ns = G.ndim >= 3 ? G.n[G.ndim - 1] : 1;
-    c.tz = G.ndim >= 3 ? tz : 1;
-    c.nchunks = G.ndim >= 3 ? (ns + c.tz - 1) / c.tz : 1;
-    return c;
 }
 
 int rows_bps(const StageParams& P, const RowsCfg& c, int dtype) {
@@ -337,70 +324,58 @@ cudaError_t rows_launch(hj_ctx* ctx, const StageParams& P0, const RowsCfg& c, in
     return dtype == HJ_F64 ? launch_rows_f64(P, c, ctx->stream) : launch_rows_f32(P, c, ctx->stream);
 }
 
-// Candidate shapes ranked by a simple cost model: whole waves of resident
-// blocks times the work of a block (warps x planes, plus one plane of
-// prologue per chunk and the halo rows per plane). The sixteen best blocks
-// with row-end threads and the eight best of n0*ty threads (the last node row
-// taking the row ends) are timed.
+// Candidate shapes ranked by a simple cost model: the work of the busiest SM
+// (blocks x warps x planes, with a plane and a half of prologue per chunk), and
+// at least the latency of its waves one after the other. The twenty best are
+// timed.
 std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtype) {
     const GridDev& G = P.g;
     const int nx = G.n[0], ny = G.n[1];
     const int D = G.ndim;
     const int ns = D >= 3 ? G.n[D - 1] : 1;
-    const size_t es = dtype == HJ_F64 ? 8 : 4;
-    static const int tys[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 16, 24, 32};
-    static const int tzs[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 128, 256};
-    std::vector<std::pair<double, RowsCfg>> scored, scored_merged;
-    for (int ty : tys) {
-        if (ty > ny || ty > nx || nx * ty > rows_max_threads(dtype == HJ_F64)) continue;
-        if (rows_smem(nx, ty, es) > 200 * 1024) continue;
-        std::vector<int> zs;
-        if (D >= 3) {
-            for (int tz : tzs)
-                if (tz < ns) zs.push_back(tz);
-            zs.push_back(ns);
-        } else {
-            zs.push_back(1);
-        }
-        for (int k = 0; k < 4 * (int)zs.size(); ++k) {
-            const int tz = zs[k / 4];
-            const bool merged = (k % 4) >= 2;  // a block of n0*ty threads: the last node row takes the row ends
-            if (!merged && (nx + 1) * ty > rows_max_threads(dtype == HJ_F64)) continue;
-            RowsCfg c = make_rows_cfg(G, ty, tz, dtype);
-            if (merged) c.nt = nx * ty;
-            if (k % 2 == 1) {  // the FP32 variant for two blocks per SM
-                if (dtype == HJ_F64 || c.nt > kRowsOcc2Threads) continue;
-                c.occ = 2;
+    const bool f64 = dtype == HJ_F64;
+    static const int tzs[] = {1, 2, 3, 4, 5, 6, 8, 10, 13, 16, 20, 24, 32, 48, 64, 128, 256};
+    static const int node_threads[] = {32, 64, 96, 128, 192, 256, 384, 512};
+    std::vector<std::pair<double, RowsCfg>> scored;
+    for (int ty : {2, 3, 4, 5, 6, 7, 8}) {
+        if (ty > ny && ty != 2) continue;
+        int last_sx = 0;
+        for (int nn : node_threads) {
+            if (nn > rows_max_node_threads(f64)) continue;
+            const int sx = rows_segment(nx, ty, nn);
+            if (sx == last_sx || (sx < 12 && sx < nx)) continue;
+            last_sx = sx;
+            for (int k = 0; k < (D >= 3 ? (int)(sizeof tzs / sizeof tzs[0]) + 1 : 1); ++k) {
+                const int tz = D < 3 ? 1 : k < (int)(sizeof tzs / sizeof tzs[0]) ? tzs[k] : ns;
+                if (D >= 3 && tz >= ns && k < (int)(sizeof tzs / sizeof tzs[0])) continue;
+                const RowsCfg c = make_rows_cfg(G, sx, ty, tz, rows_node_threads(sx, ty) + rows_edge_threads(sx));
+                if (c.nchunks > 65535 || c.nt > rows_max_threads(f64)) continue;
+                const int bps = rows_bps(P, c, dtype);
+                if (bps <= 0) continue;
+                const double blocks = (double)c.tiles * c.nchunks * (D == 4 ? G.n[2] : 1);
+                const double slots = (double)ctx->sm_count * bps;
+                const double full = std::floor(blocks / slots), rest = blocks - full * slots;
+                const double per_sm = full * bps + std::ceil(rest / ctx->sm_count);
+                const double planes = (D >= 3 ? std::min(tz, ns) : 1) + 1.5;
+                const double work = per_sm * (c.nt / 32.0) * planes;
+                const double latency = (full + (rest > 0 ? 1 : 0)) * 10.0 * planes;
+                scored.push_back({std::max(work, latency) + 0.1 * latency, c});
             }
-            if (c.nchunks > 65535 || c.row_tiles > (1 << 30)) continue;
-            const int bps = rows_bps(P, c, dtype);
-            if (bps <= 0) continue;
-            const double blocks = (double)c.row_tiles * c.nchunks * (D == 4 ? G.n[2] : 1);
-            const double slots = (double)ctx->sm_count * bps;
-            const double waves = std::ceil(blocks / slots);
-            const double warps = std::ceil((double)c.nt / 32.0);
-            const double rows_valid = std::min(ty, ny);
-            const double plane = warps * (1.0 + 0.1 * (6.0 + ty - rows_valid) / ty);
-            const double planes = D >= 3 ? (double)std::min(tz, ns) + 1.0 : 1.0;
-            (merged ? scored_merged : scored).push_back({waves * std::min((double)bps, blocks) * plane * planes, c});
         }
     }
-    const auto by_cost = [](const std::pair<double, RowsCfg>& a, const std::pair<double, RowsCfg>& b) {
-        return a.first < b.first;
-    };
-    std::sort(scored.begin(), scored.end(), by_cost);
-    std::sort(scored_merged.begin(), scored_merged.end(), by_cost);
+    std::sort(scored.begin(), scored.end(),
+              [](const std::pair<double, RowsCfg>& a, const std::pair<double, RowsCfg>& b) { return a.first < b.first; });
     std::vector<RowsCfg> out;
-    for (size_t k = 0; k < scored.size() && k < 16; ++k) out.push_back(scored[k].second);
-    for (size_t k = 0; k < scored_merged.size() && k < 8; ++k) out.push_back(scored_merged[k].second);
+    for (size_t k = 0; k < scored.size() && k < 20; ++k) out.push_back(scored[k].second);
     return out;
 }
 
 // The launch shape for this grid: measured once per (shape, dtype, dynamics,
 // scheme, dissipation) over the model's best candidates (groups of
 // first-stage launches writing to a scratch buffer, best of two groups), then
-// cached in the context. A tile override {ty, tz, occ, merged} (ty >= 1)
-// pins the shape instead; it is validated once and cached like a tuned one.
+// cached in the context. A tile override {ty, tz, occ, flags} (ty >= 1)
+// pins the rows and planes instead; it is validated once and cached like a
+// tuned shape.
 hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_t* tile, RowsCfg* out) {
     const GridDev& G = P.g;
     std::vector<long long> key = {G.ndim, P.dynamics, P.scheme, dtype, G.n[0], G.n[1], G.n[2], G.n[3],
@@ -413,15 +388,20 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
             *out = hit->second;
             return HJ_OK;
         }
-        const int ty = tile[0], tz = tile[1] > 0 ? tile[1] : 1, occ = tile[2] > 0 ? tile[2] : 1;
-        const int merged = tile[3] & 1, split = (tile[3] & 2) ? 0 : 1;
-        if (ty <= G.n[1] && ty <= G.n[0] && (G.n[0] + 1 - merged) * ty <= rows_max_threads(dtype == HJ_F64)) {
-            *out = make_rows_cfg(G, ty, tz, dtype);
-            if (merged) out->nt = G.n[0] * ty;
-            out->occ = occ;
-            out->split = split;
-            if (occ == 2 && (dtype == HJ_F64 || out->nt > kRowsOcc2Threads)) out->occ = 0;
-            if (out->occ && out->nchunks <= 65535 && rows_bps(P, *out, dtype) > 0) {
+        // which shapes fit is a matter of nodes a block (hj.h): n0 nodes by ty
+        // rows, occ 2 for FP32 blocks of up to 544 threads of one node each
+        const int tz = tile[1] > 0 ? tile[1] : 1, merged = tile[3] & 1, most = rows_max_nodes(dtype == HJ_F64);
+        const long long nx = G.n[0], want = tile[0];
+        bool fits = want <= G.n[1] && want <= nx && (nx + 1 - merged) * want <= most;
+        if (fits && tile[2] == 2) {
+            const long long one_each = nx * want + (merged ? 0 : want + (nx * want + want + nx <= most ? nx : 0));
+            fits = dtype == HJ_F32 && one_each <= 544;
+        }
+        if (fits) {
+            const int ty = std::min(tile[0], kRowsMaxTy);
+            const int sx = rows_segment(G.n[0], ty, rows_max_node_threads(dtype == HJ_F64));
+            *out = make_rows_cfg(G, sx, ty, tz, rows_node_threads(sx, ty) + rows_edge_threads(sx));
+            if (out->nchunks <= 65535 && rows_bps(P, *out, dtype) > 0) {
                 ctx->rows_cache[pkey] = *out;
                 return HJ_OK;
             }
@@ -452,9 +432,10 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
         cudaEvent_t e0, e1;
         HJ_CUDA(ctx, cudaEventCreate(&e0));
         HJ_CUDA(ctx, cudaEventCreate(&e1));
-        // FP32 launches of a few tens of microseconds are timed in groups: the
-        // event clock advances in steps of about two microseconds.
-        const int group = dtype == HJ_F64 ? 1 : (G.total < (4LL << 20) ? 6 : 2);
+        // launches of less than about 100 us are timed in groups: the event
+        // clock advances in steps of about two microseconds
+        const double per_us = dtype == HJ_F64 ? 4e3 : 4e4;  // nodes a microsecond, roughly
+        const int group = (int)std::min(8.0, std::max(1.0, std::ceil(100.0 * per_us / (double)G.total)));
         float best_ms = 1e30f;
         for (const RowsCfg& c : cands) {
             cudaError_t e = rows_launch(ctx, T, c, dtype);  // warm-up
@@ -478,28 +459,8 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
                 best = c;
             }
         }
-        // the ENO schemes: the best shape once more with interior tiles on
-        // their own body (the WENO5 kernels have no second body)
-        cudaError_t e = cudaSuccess;
-        if (P.scheme != HJ_WENO5) {
-            RowsCfg c = best;
-            c.split = 1;
-            e = rows_launch(ctx, T, c, dtype);
-            float ms_min = 1e30f;
-            for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
-                cudaEventRecord(e0, ctx->stream);
-                for (int k = 0; k < group && e == cudaSuccess; ++k) e = rows_launch(ctx, T, c, dtype);
-                cudaEventRecord(e1, ctx->stream);
-                if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-                float ms = 0.f;
-                if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
-                ms_min = std::min(ms_min, ms);
-            }
-            if (e == cudaSuccess && ms_min < best_ms) best = c;
-        }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "tuning launch");
     }
     ctx->rows_cache[key] = best;
     *out = best;

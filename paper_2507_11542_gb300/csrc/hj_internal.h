@@ -36,15 +36,17 @@ struct NvtxRange {
     NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-// Largest block of the row-tiled kernels: FP32 blocks may hold 1024 threads
-// (<= 64 registers each), FP64 blocks 512 (<= 128 registers), since the FP64
-// interface arithmetic needs more registers.
-constexpr int kRowsMaxThreadsF32 = 1024;
-constexpr int kRowsMaxThreadsF64 = 512;
-inline int rows_max_threads(int dtype_is_f64) { return dtype_is_f64 ? kRowsMaxThreadsF64 : kRowsMaxThreadsF32; }
-// The FP32 row kernel also exists compiled for two resident blocks per SM
-// (<= 56 registers a thread) of at most this many threads.
-constexpr int kRowsOcc2Threads = 544;
+// Rows of at most this many threads' worth of nodes (n0 + 1 <= 1024 in FP32,
+// 512 in FP64) are the row kernel's; a pinned launch shape may ask for up to
+// this many nodes a block.
+inline int rows_max_nodes(int dtype_is_f64) { return dtype_is_f64 ? 512 : 1024; }
+// Largest block of the row-tiled kernels, and the share its node threads may
+// take (two nodes a thread; at least one warp is left for the tile's edges):
+// FP32 blocks of 896 threads may use 72 registers a thread, FP64 blocks of 384
+// threads 168.
+constexpr int kRowsThreadsF32 = 896, kRowsThreadsF64 = 384;
+inline int rows_max_threads(int dtype_is_f64) { return dtype_is_f64 ? kRowsThreadsF64 : kRowsThreadsF32; }
+inline int rows_max_node_threads(int dtype_is_f64) { return dtype_is_f64 ? 256 : 512; }
 
 // Grid as the kernels see it. Spacing and its inverse are computed once on
 // the host from the hj_grid (periodic: (hi-lo)/n, else (hi-lo)/(n-1)).
@@ -142,37 +144,43 @@ struct UpwindParams {
 };
 
 // Launch configuration of the row-tiled stage kernel (rows_kernel.cuh).
+constexpr int kRowsMaxTy = 8;    // rows of a tile
+constexpr int kRowsMaxSx = 124;  // nodes along dimension 0 of a tile (at most four edge warps)
+constexpr int kRowsPitch = 30;  // values of one column of a shared buffer (rows_kernel.cuh says which)
 struct RowsCfg {
-    int ty;         // node rows per tile
-    int nt;         // threads per block (1-D): rows_block_threads(n0, ty, ...), or n0*ty (no row-end threads)
-    int tz;         // planes per chunk along the streamed (last) dimension
-    int nchunks;    // chunks along the streamed dimension
-    int row_tiles;  // ceil(n1 / ty)
-    int occ;        // 1, or 2: FP32 kernel compiled for two resident blocks of <= kRowsOcc2Threads threads per SM
-    int split;      // 1: interior tiles take the body compiled without ghost and wrap logic (ENO schemes)
+    int sx;       // nodes along dimension 0 of a tile
+    int ty;       // node rows per tile, at most kRowsMaxTy
+    int nt;       // threads per block (1-D), a multiple of 32
+    int tz;       // planes per chunk along the streamed (last) dimension
+    int nchunks;  // chunks along the streamed dimension
+    int tiles;    // ceil(n0 / sx) * ceil(n1 / ty)
 };
-
-// Threads of a row-kernel block with ty node rows of n0 nodes: one thread per
-// node, one per row for the row's last dimension-0 interface and ghost cells,
-// and, where the block size allows it, one per column for the tile's last
-// dimension-1 interface (without them thread row 0 evaluates those).
-inline bool rows_gap_threads(int nx, int ty, int threads) { return nx * ty + ty + nx <= threads; }
-inline int rows_block_threads(int nx, int ty, int max_threads) {
-    return nx * ty + ty + (rows_gap_threads(nx, ty, max_threads) ? nx : 0);
+// threads of the node warps (two rows each)
+__host__ __device__ inline int rows_node_threads(int sx, int ty) { return (sx * ((ty + 1) / 2) + 31) / 32 * 32; }
+__host__ __device__ inline int rows_buf_elems(int sx) { return (sx + 6) * kRowsPitch; }
+// Dynamic shared memory of a block (element size es).
+inline size_t rows_smem(int sx, size_t es) { return 2 * es * (size_t)rows_buf_elems(sx); }
+// The widest segment (nodes along dimension 0, as equal as possible) with which
+// ty rows of n0 nodes fit node_threads node threads.
+inline int rows_segment(int n0, int ty, int node_threads) {
+    const int fit = node_threads / ((ty + 1) / 2);
+    const int most = fit < kRowsMaxSx ? fit : kRowsMaxSx;
+    const int nseg = (n0 + most - 1) / most;
+    return (n0 + nseg - 1) / nseg;
 }
-
-// Elements of one of the two alternating shared buffers of a rows_kernel
-// block: (ty + 6) padded rows of n0 + 6, then p+ along dimension 0 (ty rows
-// of n0 + 1), along dimension 1 (ty + 1 rows of n0), and the two outermost
-// values at each end of every node row (4 per row, for the ghost cells).
-__host__ __device__ inline size_t rows_buf_elems(int nx, int ty) {
-    return (size_t)(ty + 6) * (size_t)(nx + 6) + (size_t)ty * (size_t)(nx + 1) + (size_t)(ty + 1) * (size_t)nx +
-           4 * (size_t)ty;
-}
-
-// Dynamic shared memory of a rows_kernel block (element size es).
-inline size_t rows_smem(int nx, int ty, size_t es) {
-    return 2 * es * rows_buf_elems(nx, ty);
+// Edge threads beside a tile's node threads: one per column and row pair (their
+// last interfaces, and the halo of their line).
+inline int rows_edge_threads(int sx) { return (sx + 4 + 31) / 32 * 32; }
+inline RowsCfg make_rows_cfg(const GridDev& G, int sx, int ty, int tz, int nt) {
+    RowsCfg c;
+    c.sx = sx;
+    c.ty = ty;
+    c.nt = nt;
+    c.tiles = ((G.n[0] + sx - 1) / sx) * ((G.n[1] + ty - 1) / ty);
+    const int ns = G.ndim >= 3 ? G.n[G.ndim - 1] : 1;
+    c.tz = G.ndim >= 3 ? tz : 1;
+    c.nchunks = (ns + c.tz - 1) / c.tz;
+    return c;
 }
 
 // Launchers (one translation unit per element type). Return the launch error.
@@ -196,14 +204,14 @@ int rows_blocks_per_sm_f32(const StageParams& p, const RowsCfg& c);
 // ---------------------------------------------------------------------------
 struct BatchTile {
     int inst;      // instance index
-    int row_tile;  // rows row_tile*ty .. of the instance's planes
+    int tile;      // tile of the instance's planes: segment + segments * row tile
     int i2;        // dimension-2 index (4-D instances)
     int chunk;     // chunk along the streamed dimension
 };
 
 struct BatchInst {
     StageParams P;            // grid, dynamics, parameters (FP64 + FP32), angle tables, WENO floor
-    int ty, tz;               // tile shape of this instance
+    int sx, ty, tz;           // tile shape of this instance
     int steps_total;          // RK3 steps of the whole solve
     int k;                    // steps completed (advanced on the device)
     double dt;                // dt of the current step

@@ -1,25 +1,26 @@
 // rows_kernel.cuh -- the fused RK stage kernel (WENO5, ENO1/2/3) on 2-4 dimensional
 // grids, tiled for GB300:
 //
-//  * A thread block (1-D) owns TY full rows (all n0 nodes along dimension 0)
-//    of one plane of dimensions (0, 1): one thread per node, one per row end
-//    and, where the block has room, one per column for the tile's last
-//    dimension-1 interface, each role in its own warps. The plane with
-//    three halo rows above and below lives in shared memory.
+//  * A thread block owns a tile of one plane of dimensions (0, 1): a segment of
+//    SX nodes along dimension 0 by TY <= 8 rows, with three halo cells on each
+//    side. Each node thread works on two neighbouring rows of its column (one
+//    per lane of a pair, lanes.cuh): one walk through addresses, predicates and
+//    loop control serves two nodes, and FP32 arithmetic is packed.
 //  * The upwind scheme (WENO5, ENO1/2/3) is evaluated per interface (one
 //    interface gives p+ of a node and p- of the next). Along dimension 0 the
-//    node thread x computes the interface between nodes x-1 and x (the row
-//    end the row's last one); along dimension 1 the node thread of row k the
-//    one between tile rows k-1 and k (the gap threads the tile's last one).
-//    So each node pays for about one interface per dimension instead of two.
+//    node thread of column x computes the interfaces between x-1 and x of its
+//    two rows; along dimension 1 the one below its first row and the one
+//    between its two rows. So each node pays for about one interface per
+//    dimension instead of two.
+//  * Whole warps have one role: node warps hold the node threads; edge warps
+//    copy the halos two planes ahead and compute what is left over at the
+//    tile's edges (the last interface of every row, the gap above the last row).
 //  * For 3-D and 4-D grids the block streams along the last dimension through
-//    a chunk of planes: each thread keeps six values of its column in
-//    registers and carries the interface result p- to the next plane. Planes
-//    are staged in shared memory two ahead of their use (asynchronous
-//    copies), with one barrier per plane.
+//    a chunk of planes: each thread keeps its columns' values in registers and
+//    carries the interface result p- to the next plane. One barrier per plane.
 //  * In 4-D, dimension 2 is differentiated two-sided from 7-point loads.
 //  * Ghost values (periodic wrap or slope continued away from zero, Sec. 2.1)
-//    are produced where values are read; no padded array exists.
+//    are produced where values are staged; no padded array exists.
 // Then: Hamiltonian + Lax-Friedrichs dissipation (Sec. 4), BRT clamp (Sec.
 // 6.1) and the TVD-RK3 stage combination (Sec. 5), one store per node.
 #pragma once
@@ -33,32 +34,17 @@
 namespace hj {
 
 template <typename T> struct RowsLimits;
-template <> struct RowsLimits<float> { static constexpr int kMaxThreads = kRowsMaxThreadsF32; };
-template <> struct RowsLimits<double> { static constexpr int kMaxThreads = kRowsMaxThreadsF64; };
-// Launch bounds of a row-kernel variant: OCC resident blocks per SM.
-template <typename T, int OCC> struct RowsBounds {
-    static constexpr int kThreads = OCC == 2 ? kRowsOcc2Threads : RowsLimits<T>::kMaxThreads;
-};
+template <> struct RowsLimits<float> { static constexpr int kThreads = kRowsThreadsF32; };
+template <> struct RowsLimits<double> { static constexpr int kThreads = kRowsThreadsF64; };
 
+// The slope that ghost values continue outward, and the m-th ghost value.
+template <typename T>
+__device__ __forceinline__ T outward_slope(T edge, T inner, int extrap) {
+    return (extrap == HJ_EXTRAP_LINEAR) ? (edge - inner) : fabs(edge - inner) * sgn(edge);
+}
 template <typename T>
 __device__ __forceinline__ T ghost_value(T edge, T inner, int m, int extrap) {
-    const T s = (extrap == HJ_EXTRAP_LINEAR) ? (edge - inner) : fabs(edge - inner) * sgn(edge);
-    return add_rn(edge, mul_rn(T(m), s));
-}
-
-// Value at index i of a grid line (base pointer, n nodes, stride s), with the
-// line's ghost rule outside [0, n).
-template <typename T>
-__device__ __forceinline__ T line_value(const T* __restrict__ base, int i, int n, long long s, bool periodic,
-                                        int extrap) {
-    if (i >= 0 && i < n) return ld(base + (long long)i * s);
-    if (periodic) {
-        int j = i % n;
-        if (j < 0) j += n;
-        return ld(base + (long long)j * s);
-    }
-    if (i < 0) return ghost_value(ld(base), ld(base + s), -i, extrap);
-    return ghost_value(ld(base + (long long)(n - 1) * s), ld(base + (long long)(n - 2) * s), i - (n - 1), extrap);
+    return add_rn(edge, mul_rn(T(m), outward_slope(edge, inner, extrap)));
 }
 
 // Values of one stage launch that differ between the three RK stages, in the
@@ -105,449 +91,438 @@ template <> __device__ __forceinline__ void cp_async_elem<double>(double* dst, c
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 
-// One tile: rows y0 = row_tile*TY .. +TY-1 of the plane(s) at dimension-2 index
-// i2 (4-D) and the planes of chunk `chunk` along the streamed dimension
-// (planes chunk*tz .. +tz-1), computed by the NT threads of a 1-D block.
-// Thread t has one role, so that roles change only between whole warps
-// (except one warp at each boundary):
-//   t <  n0*TY          node (x, r) = (t mod n0, t div n0);
-//   t <  n0*TY + TY     row end of row r = t - n0*TY (x = n0);
-//   t <  n0*TY+TY+n0    gap thread of column x (present when the block has
-//                       room: NT >= n0*TY + TY + n0);
-//   others              barriers only.
-// A block of exactly n0*TY threads has no row-end threads: node thread x of
-// the last node row takes the end of row x as well (rows of n0 >= TY nodes).
-//
-// Interfaces along dimensions 0 and 1 are each evaluated once per plane and
-// shared through shared memory:
-//   x-interfaces: node (x, r) takes the one between nodes x-1 and x, the row
-//                 end the row's last one;
-//   y-interfaces: node (x, r) takes gap r (between tile rows r-1 and r), the
-//                 gap thread of column x the tile's last gap (without gap
-//                 threads: an idle node row of a ragged tile, else row 0).
-// The p- half of the interface a thread evaluates for its own node stays in a
-// register; the p+ half belongs to the neighbour (x-1 or row r-1) and goes
-// through shared memory. Derivatives stay raw (undivided differences) until
-// the node combines them, scaled by 1/(2 dx), into the means and half
-// differences the Hamiltonian takes.
-//
-// Planes are software-pipelined through two shared buffers (plane p in
-// buffer p mod 2) with one barrier per plane:
-//   phase A(z): interfaces of plane z; ghost cells of plane z+1 from its row
-//               ends; wait for this thread's copies into plane z+1
+__device__ __forceinline__ void block_barrier(int threads) { asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory"); }
+
+// Where a tile lies and who works on it (the same for all threads of a block).
+struct Tile {
+    int x0, sx;     // first node of the segment along dimension 0, nodes in it
+    int y0, rv;     // first row, rows in the grid
+    int i2;         // dimension-2 index (4-D)
+    int zbeg, zend; // planes along the streamed dimension
+    int stride;     // SX: node thread t works on column t mod SX, row pair t div SX
+    int nn, nt;     // threads of the node warps, all threads
+};
+
+// Shared memory: two buffers (plane p in buffer (p - zbeg) mod 2), each a column
+// of kPitch values per node of the segment and three more on each side:
+//   [0, 16)   rows -4 .. 11 of the plane (row r at 4 + r; -4 and 11 unused)
+//   [16, 24)  p+ of the node to the left along dimension 0, per row
+//   [24, 29)  p+ of row 2k - 1 along dimension 1
+// so that both neighbour directions are constant offsets from one address, and
+// a thread's two rows are one aligned access. A pitch of 30 spreads a warp's
+// pairs over all banks.
+constexpr int kColX = 16, kColY = 24;
+
+// One tile. Planes are software-pipelined with one barrier per plane:
+//   phase A(z): interfaces of plane z along dimensions 0 and 1 (node and edge
+//               warps); edge warps wait for their copies into plane z+1
 //   barrier
-//   phase B(z): node updates of plane z; staging of plane z+2 (node values
-//               from the column queues, halo rows and row ends copied
-//               asynchronously), two planes ahead of its use.
-// Flat indices are 32-bit (the grid has fewer than 2^31 nodes).
-//
-// IN: the tile is interior (all TY rows in the grid, its halo rows and the
-// chunk's streamed-dimension reads inside the grid): no ghost or wrap logic
-// is compiled for its staging and queue loads (a block-uniform dispatch).
-template <typename T, int D, int DYN, int SCHEME, int KIND, bool IN = false>
-__device__ __forceinline__ void rows_tile(const StageParams& P, const StageRun<T>& R, const int TY, const int NT,
-                                          const int tz, const int row_tile, const int i2_in, const int chunk_in,
-                                          const int t, T* const smem) {
+//   phase B(z): node updates of plane z; staging of plane z+2 (node values from
+//               the column queues, halos by the edge warps' asynchronous copies)
+// The p- half of an interface stays in a register, the p+ half goes through
+// shared memory where another thread owns the node. Derivatives stay raw
+// (undivided differences) until the node combines them, scaled by 1/(2 dx),
+// into the means and half differences the Hamiltonian takes. Flat indices are
+// 32-bit (the grid has fewer than 2^31 nodes). Threads of the node warps
+// without a node work on a clamped one and store nothing.
+template <typename T, int D, int SCHEME>
+__device__ __forceinline__ void edge_warps(const StageParams& P, const T* __restrict__ u, const Tile& C, const int t,
+                                           T* const smem, const int buf) {
+    constexpr int kP = kRowsPitch;
+    constexpr int SD = (D >= 3) ? D - 1 : 0;
     const GridDev& g = P.g;
     const int nx = g.n[0], ny = g.n[1];
-    const int W = nx + 6;  // shared row: 3 ghost cells, nx nodes, 3 ghost cells
-    // per buffer: (TY + 6) rows x W, p+ along dimension 0 (TY rows of nx + 1),
-    // p+ along dimension 1 (TY + 1 rows of nx), row ends (4 per node row)
-    const int buf_elems = (int)rows_buf_elems(nx, TY);
-    const int o_pxp = (TY + 6) * W;
-    const int o_pyp = o_pxp + TY * (nx + 1);
-    const int o_ends = o_pyp + (TY + 1) * nx;
+    const bool per0 = g.periodic_mask & 1u, per1 = (g.periodic_mask >> 1) & 1u;
+    const int extrap = g.extrap;
+    const int et = t - C.nn, en = C.nt - C.nn;
+    const int sS = (D >= 3) ? (int)g.stride[SD] : 0;
+    const int plane0 = (D == 4) ? C.i2 * (int)g.stride[2] : 0;
+    const T fl0 = SP<T>::floor(P, 0), fl1 = SP<T>::floor(P, 1);
 
+    // A thread's share of a plane's halo (en >= sx + 4): the rows -3, -2, -1, rv,
+    // rv+1, rv+2 of column et, and for the last eight threads the columns -3,
+    // -2, -1, sx, sx+1, sx+2 of a row. Sources do not change from plane to plane:
+    // a flat index of plane 0, or the distance of a ghost cell from the grid
+    // (extrapolated edges). A ghost cell needs the two outermost values at its
+    // end of the line, which are loaded one plane before they are used.
+    struct Line {
+        int src[6];        // flat index, or -1: a ghost cell
+        T m[6];            // ghost cell: its distance from the grid
+        int lo0, lo1, hi0, hi1;
+        bool lo, hi;       // the line has ghost cells below, above
+        T a0, a1, b0, b1;  // its outermost values in the next plane
+    };
+    auto make_line = [&](Line& l, int first, int last, int n, bool periodic, int base, int step) {
+        l.lo = l.hi = false;
+        l.a0 = l.a1 = l.b0 = l.b1 = T(0);
+        l.lo0 = base;
+        l.lo1 = base + step;
+        l.hi0 = base + (n - 1) * step;
+        l.hi1 = base + (n - 2) * step;
+#pragma unroll
+        for (int h = 0; h < 6; ++h) {
+            int i = h < 3 ? first + h - 3 : last + h - 3;  // -3 .. n + 2
+            const bool below = i < 0, above = i >= n;
+            if (periodic) i += below ? n : above ? -n : 0;
+            else if (below) l.lo = true;
+            else if (above) l.hi = true;
+            const bool ghost = !periodic && (below || above);
+            l.src[h] = ghost ? -1 : base + i * step;
+            l.m[h] = T(below ? -i : i - (n - 1));
+        }
+    };
+    auto fetch = [&](Line& l, int p) {
+        const T* __restrict__ plane = u + p * sS;
+        if (l.lo) { l.a0 = ld(plane + l.lo0); l.a1 = ld(plane + l.lo1); }
+        if (l.hi) { l.b0 = ld(plane + l.hi0); l.b1 = ld(plane + l.hi1); }
+    };
+    auto put = [&](const Line& l, int p, T* low, T* high, int step) {
+        const T* __restrict__ plane = u + p * sS;
+        const T sa = outward_slope(l.a0, l.a1, extrap), sb = outward_slope(l.b0, l.b1, extrap);
+#pragma unroll
+        for (int h = 0; h < 6; ++h) {
+            T* dst = h < 3 ? low + h * step : high + (h - 3) * step;
+            if (l.src[h] >= 0) cp_async_elem(dst, plane + l.src[h]);
+            else *dst = add_rn(h < 3 ? l.a0 : l.b0, mul_rn(l.m[h], h < 3 ? sa : sb));
+        }
+    };
+    const bool col_job = et < C.sx;
+    const int r = et - (en - kRowsMaxTy);
+    const bool row_job = r >= 0 && r < C.rv;
+    Line col, row;
+    if (col_job) make_line(col, C.y0, C.y0 + C.rv, ny, per1, plane0 + C.x0 + et, nx);
+    if (row_job) make_line(row, C.x0, C.x0 + C.sx, nx, per0, plane0 + (C.y0 + r) * nx, 1);
+    auto fetch_all = [&](int p) {
+        if (col_job) fetch(col, p);
+        if (row_job) fetch(row, p);
+    };
+    auto stage = [&](int p, T* b) {
+        if (col_job) put(col, p, b + (et + 3) * kP + 1, b + (et + 3) * kP + 4 + C.rv, 1);
+        if (row_job) put(row, p, b + 4 + r, b + (C.sx + 3) * kP + 4 + r, kP);
+        if (p + 1 < C.zend) fetch_all(p + 1);
+    };
+
+    fetch_all(C.zbeg);
+    stage(C.zbeg, smem);
+    if (C.zbeg + 1 < C.zend) stage(C.zbeg + 1, smem + buf);
+    cp_async_wait_all();
+    block_barrier(C.nt);
+
+    // left-over interfaces: the gap above the last row where no node thread has
+    // it (an even number of rows), then the last one of each row pair
+    const int n_gap = (C.rv & 1) ? 0 : C.sx;
+    const int n_item = n_gap + ((C.rv + 1) >> 1);
+#pragma unroll 1
+    for (int z = C.zbeg; z < C.zend; ++z) {
+        T* const bz = smem + ((z - C.zbeg) & 1) * buf;
+#pragma unroll 1
+        for (int i = et; i < n_item; i += en) {
+            const bool gap = i < n_gap;
+            const int pr = i - n_gap;
+            const T* w0 = gap ? bz + (i + 3) * kP + 1 + C.rv : bz + C.sx * kP + 4 + 2 * pr;
+            const int step = gap ? 1 : kP, second = gap ? 0 : 1;
+            Lanes<T> w[6], pp, pm;
+#pragma unroll
+            for (int k = 0; k < 6; ++k) w[k] = lanes(w0[k * step], w0[k * step + second]);
+            iface_lanes<SCHEME>(w, gap ? fl1 : fl0, pp, pm);
+            if (gap) bz[(i + 3) * kP + kColY + (C.rv >> 1)] = lane_a(pp);
+            else put_lanes(bz + (C.sx + 3) * kP + kColX + 2 * pr, pp);
+        }
+        cp_async_wait_all();  // this thread's copies into plane z+1
+        block_barrier(C.nt);
+        if (z + 2 < C.zend) stage(z + 2, bz);
+    }
+}
+
+template <typename T, int D, int DYN, int SCHEME, int KIND>
+__device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<T>& R, const Tile& C, const int t,
+                                           T* const smem, const int buf) {
+    using L = Lanes<T>;
+    constexpr int kP = kRowsPitch;
+    constexpr int SD = (D >= 3) ? D - 1 : 0;  // streamed dimension
+    const GridDev& g = P.g;
+    const int nx = g.n[0], ny = g.n[1];
     const T* __restrict__ u = R.u;
     const T* __restrict__ vn = R.vn;
     T* __restrict__ out = R.out;
-    const bool per0 = g.periodic_mask & 1u, per1 = (g.periodic_mask >> 1) & 1u;
-    const int extrap = g.extrap;
+    T* __restrict__ also_out = R.also_out;
 
-    const int y0 = row_tile * TY;
-    const int rows_valid = min(TY, ny - y0);
-    // roles
-    const int n_node = nx * TY;
-    const int n_end = n_node + TY;
-    const bool gaps = nx * TY + TY + nx <= NT;
-    const bool is_node = t < n_node;
-    const bool is_end = t >= n_node && t < n_end;
-    const bool is_gap = gaps && t >= n_end && t < n_end + nx;
-    int x, r;
-    if (is_node) {
-        r = t / nx;
-        x = t - r * nx;
-    } else if (is_end) {
-        r = t - n_node;
-        x = nx;
-    } else {
-        r = TY;
-        x = is_gap ? t - n_end : nx;
-    }
-    const int y = y0 + r;
-    const bool node = is_node && r < rows_valid;
-    const bool do_xrow = (is_node || is_end) && r < rows_valid;
-    // this thread's gap (tile row boundary) along dimension 1, or -1
-    int gk = -1;
-    if (is_node && r < rows_valid) gk = r;
-    else if (is_gap) gk = rows_valid;
-    else if (!gaps && is_node && r == rows_valid) gk = rows_valid;  // an idle row of a ragged tile
-    const bool do_ylast = !gaps && rows_valid == TY && is_node && r == 0;  // full tile, no gap threads
-    // The row-end role of a tile row er: the row's last dimension-0 interface,
-    // its ghost sources and ghost cells. Row-end threads take it, or, in a
-    // block of exactly n0*TY threads (no row-end threads), node thread x of the
-    // last node row takes the end of row x: that row's threads evaluate one
-    // interface fewer than row 0's, which also takes the tile's last gap.
-    const bool merged = NT < n_end;
-    const bool spare = merged ? (is_node && r == TY - 1 && x < rows_valid) : (is_end && r < rows_valid);
-    const int er = merged ? x : r;
-    const int ey = y0 + er;
+    int pr = t / C.stride, x = t - pr * C.stride;
+    const bool node = x < C.sx && 2 * pr < C.rv;      // this thread's first row
+    const bool node1 = node && 2 * pr + 1 < C.rv;      // its second
+    x = min(x, C.sx - 1);
+    pr = min(pr, (C.rv - 1) >> 1);
+    const int y = C.y0 + 2 * pr;
+    const int y1 = min(y + 1, ny - 1);
 
-    const int i2 = (D == 4) ? i2_in : 0;
-    const int chunk = (D >= 3) ? chunk_in : 0;
-    constexpr int SD = (D >= 3) ? D - 1 : 0;  // streamed dimension
-    const T fl0 = SP<T>::floor(P, 0), fl1 = SP<T>::floor(P, 1), flS = SP<T>::floor(P, SD);
     const int ns = (D >= 3) ? g.n[SD] : 1;
-    const int zbeg = (D >= 3) ? chunk * tz : 0;
-    const int zend = (D >= 3) ? min(ns, zbeg + tz) : 1;
     const int sS = (D >= 3) ? (int)g.stride[SD] : 0;
     const bool perS = (D >= 3) ? ((g.periodic_mask >> SD) & 1u) : false;
-    // the chunk's streamed-dimension reads stay inside the grid: no ghost logic needed
-    const bool z_inside = IN || (D < 3) || (zbeg >= 3 && zend + 3 <= ns);
-    const int plane0 = (D == 4) ? i2 * (int)g.stride[2] : 0;      // flat index of (0, 0, i2, 0)
-    const int col = plane0 + min(x, nx - 1) + min(y, ny - 1) * nx;  // flat index of (x, y) at streamed index 0
-    const T* __restrict__ ucol = u + col;
+    const int extrap = g.extrap;
+    const int plane0 = (D == 4) ? C.i2 * (int)g.stride[2] : 0;
+    const int col0 = plane0 + C.x0 + x + y * nx;   // flat index of the first row's node at streamed index 0
+    const int col1 = plane0 + C.x0 + x + y1 * nx;
+    const T fl0 = SP<T>::floor(P, 0), fl1 = SP<T>::floor(P, 1), flS = SP<T>::floor(P, SD);
 
-    // shared-memory offsets within a buffer
-    const int s_center = (r + 3) * W + 3 + x;
-    const int s_xrow = (r + 3) * W + x;        // value at node x - 3 of row r
-    const int s_ycol = gk * W + 3 + x;         // value at tile row gk - 3 of column x
-    const int s_ylast = TY * W + 3 + x;
-    const int s_pxp = o_pxp + r * (nx + 1) + x;  // p+ of node x - 1 of row r (written); + 1: of node x (read)
-    const int s_pyw = o_pyp + gk * nx + x;       // p+ of tile row gk - 1 (written)
-    const int s_pyr = o_pyp + (r + 1) * nx + x;  // p+ of tile row r (read)
+    // values of both columns at plane z (z within three of the grid; ns >= 4)
+    auto column = [&](int z) -> L {
+        if (z >= 0 && z < ns) return lanes(ld(u + col0 + z * sS), ld(u + col1 + z * sS));
+        if (perS) {
+            const int w = z + (z < 0 ? ns : -ns);
+            return lanes(ld(u + col0 + w * sS), ld(u + col1 + w * sS));
+        }
+        const int e = z < 0 ? 0 : ns - 1, i = z < 0 ? 1 : ns - 2, m = z < 0 ? -z : z - (ns - 1);
+        return lanes(ghost_value(ld(u + col0 + e * sS), ld(u + col0 + i * sS), m, extrap),
+                     ghost_value(ld(u + col1 + e * sS), ld(u + col1 + i * sS), m, extrap));
+    };
 
     // 1/(2 dx), or 1/(12 dx) where the interface evaluation returns six times the derivatives
     const auto half_inv = [&P](int d) -> T {
         if constexpr (iface_times6<T, SCHEME>()) return SP<T>::half_inv_dx6(P, d);
         else return SP<T>::half_inv_dx(P, d);
     };
-    const T h0 = half_inv(0), h1 = half_inv(1), hS = half_inv(SD);
-    const T dt = R.dt, cv = R.cv, cu = R.cu;
-    const bool minv = R.minv;
-    // BRT min(0, .) as a clamp (+inf: none), global dissipation as a flag, both read once
-    const bool brt0 = R.brt0;
-    const T clamp = brt0 ? T(0) : T(INFINITY);
-    const bool alpha_global = P.alpha_global;
-    T* __restrict__ also_out = R.also_out;
-    // node coordinates that do not change along the streamed dimension
-    T xc[D];
+    T hh[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) xc[d] = T(0);
-    if constexpr (uses_coord<D, DYN>(0)) xc[0] = coord(SP<T>::lo(P, 0), x, SP<T>::dx(P, 0));
-    if constexpr (uses_coord<D, DYN>(1)) xc[1] = coord(SP<T>::lo(P, 1), y, SP<T>::dx(P, 1));
-    if constexpr (D == 4 && uses_coord<D, DYN>(2)) xc[2] = coord(SP<T>::lo(P, 2), i2, SP<T>::dx(P, 2));
+    for (int d = 0; d < D; ++d) hh[d] = half_inv(d);
+    const T dt = R.dt, cv = R.cv, cu = R.cu;
+    const bool minv = R.minv, brt0 = R.brt0;
+    const T clamp = brt0 ? T(0) : T(INFINITY);  // BRT min(0, .) as a clamp (+inf: none)
+    const bool alpha_global = P.alpha_global;
+    // node coordinates that do not change along the streamed dimension
+    T xa[D], xb[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) xa[d] = xb[d] = T(0);
+    if constexpr (uses_coord<D, DYN>(0)) xa[0] = xb[0] = coord(SP<T>::lo(P, 0), C.x0 + x, SP<T>::dx(P, 0));
+    if constexpr (uses_coord<D, DYN>(1)) {
+        xa[1] = coord(SP<T>::lo(P, 1), y, SP<T>::dx(P, 1));
+        xb[1] = coord(SP<T>::lo(P, 1), y1, SP<T>::dx(P, 1));
+    }
+    if constexpr (D == 4 && uses_coord<D, DYN>(2)) xa[2] = xb[2] = coord(SP<T>::lo(P, 2), C.i2, SP<T>::dx(P, 2));
     const T* __restrict__ trig = Trig<T>::get(P);       // cos of the dimension-2 coordinate
     const T* __restrict__ trig_s = uses_angle<D, DYN>() ? trig + g.n[2] : trig;  // sin
-    T cos2 = T(0), sin2 = T(0);  // angle of dimension 2 (fixed for the block in 4-D)
+    T cos2 = T(0), sin2 = T(0);  // angle of dimension 2 (fixed for the block in 4-D, the next plane's in 3-D)
     if constexpr (D == 4 && uses_angle<D, DYN>()) {
-        cos2 = trig[i2];
-        sin2 = trig_s[i2];
+        cos2 = trig[C.i2];
+        sin2 = trig_s[C.i2];
     }
-
-    // Halo rows (three above, three below, and rows past the grid edge in a
-    // ragged last tile): slot s = h * nx + hx of the n_extra * nx halo values
-    // goes to thread s, s - NT, ... (node threads take their own column).
-    const int n_extra = 3 + (TY + 3 - rows_valid);
-    const int n_halo = n_extra * nx;
-
-    // Plane p into buffer b, except the node values: halo rows (in-grid or
-    // periodic rows copied asynchronously, rows past an extrapolated edge by
-    // the ghost rule) and, from the row ends, the row's x-ghost sources
-    // (periodic: the wrapped nodes into the ghost cells; extrapolated: the
-    // two outermost nodes at each end into the row-end slots).
-    auto halo_slot = [&](int sidx, int fp, T* b) {
-        const int h = sidx / nx, hx = sidx - h * nx;
-        const int rr = (h < 3) ? h - 3 : rows_valid + (h - 3);
-        int yy = y0 + rr;
-        T* dst = b + (rr + 3) * W + 3 + hx;
-        if (!IN && per1 && (yy < 0 || yy >= ny)) yy = (yy % ny + ny) % ny;
-        const T* base = u + plane0 + fp + hx;
-        if (IN || (yy >= 0 && yy < ny)) cp_async_elem(dst, base + yy * nx);
-        else *dst = line_value(base, yy, ny, (long long)nx, false, extrap);
-    };
-    // this thread's first halo slot (the same in every plane): destination and source
-    const bool h0_on = t < n_halo;
-    const int h0_h = t / nx, h0_x = t - (t / nx) * nx;
-    const int h0_rr = (h0_h < 3) ? h0_h - 3 : rows_valid + (h0_h - 3);
-    const int h0_dst = (h0_rr + 3) * W + 3 + h0_x;
-    int h0_yy = y0 + h0_rr;
-    if (!IN && per1 && (h0_yy < 0 || h0_yy >= ny)) h0_yy = (h0_yy % ny + ny) % ny;
-    const bool h0_in = IN || (h0_yy >= 0 && h0_yy < ny);
-    const int h0_src = plane0 + h0_x + (h0_in ? h0_yy * nx : 0);
-    auto stage_rest = [&](int p, T* b) {
-        const int fp = p * sS;
-        if (h0_on) {
-            if (h0_in) cp_async_elem(b + h0_dst, u + h0_src + fp);
-            else b[h0_dst] = line_value(u + plane0 + fp + h0_x, h0_yy, ny, (long long)nx, false, extrap);
-        }
-        for (int sidx = t + NT; sidx < n_halo; sidx += NT) halo_slot(sidx, fp, b);  // small blocks, ragged tiles
-        if (spare) {
-            const T* rowg = u + plane0 + fp + ey * nx;
-            if (per0) {
-                T* rows = b + (er + 3) * W;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    cp_async_elem(rows + k, rowg + nx - 3 + k);
-                    cp_async_elem(rows + nx + 3 + k, rowg + k);
-                }
-            } else {
-                T* e = b + o_ends + 4 * er;
-                cp_async_elem(e + 0, rowg);
-                cp_async_elem(e + 1, rowg + 1);
-                cp_async_elem(e + 2, rowg + nx - 1);
-                cp_async_elem(e + 3, rowg + nx - 2);
-            }
-        }
-    };
-    // Row end, after its copies into b have landed: the extrapolated x-ghost cells of its row.
-    auto finish_ghosts = [&](T* b) {
-        if (spare && !per0) {
-            const T* e = b + o_ends + 4 * er;
-            T* rows = b + (er + 3) * W;
-            const T e0 = e[0], e1 = e[1], f0 = e[2], f1 = e[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                rows[k] = ghost_value(e0, e1, 3 - k, extrap);
-                rows[nx + 3 + k] = ghost_value(f0, f1, k + 1, extrap);
-            }
-        }
-    };
-
+    if constexpr (D == 3 && uses_angle<D, DYN>()) {
+        cos2 = trig[C.zbeg];
+        sin2 = trig_s[C.zbeg];
+    }
 
     // Streamed-dimension queue: q[k] = V at plane z-2+k (k = 0..5); carry = raw p- at z.
     // A warm-up step evaluates the interface below the first plane, so that
     // every interface goes through the same code and results do not depend
-    // on where chunks start.
-    // In FP64 WENO5 the streamed-dimension interfaces slide along the column:
-    // each reuses the differences of the one below it (Weno5Line, bit for bit
-    // the same results as a full evaluation).
+    // on where chunks start. FP64 WENO5 keeps the differences instead
+    // (Weno5Line, bit for bit the same results).
     constexpr bool kSlide = std::is_same<T, double>::value && SCHEME == HJ_WENO5 && D >= 3;
-    T q[6];
-    T carry = T(0);
-    Weno5Line zline;
-    if (D >= 3 && node) {
+    L q[6], q6{}, carry{};
+    Weno5Line za, zb;
+    if constexpr (D >= 3) {
 #pragma unroll
-        for (int k = 0; k < 6; ++k)
-            q[k] = IN ? ld(ucol + (zbeg - 3 + k) * sS) : line_value(ucol, zbeg - 3 + k, ns, (long long)sS, perS, extrap);
-        T unused;
+        for (int k = 0; k < 6; ++k) q[k] = column(C.zbeg - 3 + k);
+        L unused;
         if constexpr (kSlide) {
-            zline.start(q[0], q[1], q[2], q[3], q[4], q[5]);
-            zline.eval(flS, unused, carry);
+            za.start(q[0].a, q[1].a, q[2].a, q[3].a, q[4].a, q[5].a);
+            za.eval(flS, unused.a, carry.a);
+            zb.start(q[0].b, q[1].b, q[2].b, q[3].b, q[4].b, q[5].b);
+            zb.eval(flS, unused.b, carry.b);
         } else {
-            iface_at<SCHEME>(q[0], q[1], q[2], q[3], q[4], q[5], flS, unused, carry);
+            iface_lanes<SCHEME>(q, flS, unused, carry);
         }
 #pragma unroll
         for (int k = 0; k < 5; ++k) q[k] = q[k + 1];
+        q6 = column(C.zbeg + 3);
+    } else {
+        q[2] = column(0);
     }
 
-    // V^n of the node's next plane is loaded one plane ahead of its use (2-D
-    // and 3-D grids), so that its global-memory latency is covered by a whole
-    // plane of work. Where out aliases V^n, the value read is this thread's own
-    // node, which it writes one plane later.
+    // The queue's next value, the next angle and V^n of the next plane (2-D and
+    // 3-D grids) are loaded one plane ahead of their use, so that a whole plane
+    // of work covers their latency. Where out aliases V^n, the value read is
+    // this thread's own node, which it writes one plane later.
     constexpr bool kVnAhead = KIND == kKindCombine && D <= 3;
-    T vn_next = T(0);
+    int f0 = col0 + C.zbeg * sS, f1 = col1 + C.zbeg * sS;  // the two nodes of plane z
+    const T* __restrict__ u4 = u + 4 * (long long)sS;
+    const T* __restrict__ vn_next = vn + sS;
+    T vn0 = T(0), vn1 = T(0);
     if constexpr (kVnAhead) {
-        if (node) vn_next = ld(vn + col + zbeg * sS);
+        vn0 = ld(vn + f0);
+        vn1 = ld(vn + f1);
     }
 
-    // prologue: planes zbeg and zbeg+1 (ghost cells of zbeg+1 follow in phase A(zbeg))
-    {
-        T* const b0 = smem;
-        if (node) b0[s_center] = (D >= 3) ? q[2] : ld(ucol);
-        stage_rest(zbeg, b0);
-        if (zbeg + 1 < zend) {
-            T* const b1 = smem + buf_elems;
-            if (node) b1[s_center] = q[3];
-            stage_rest(zbeg + 1, b1);
-        }
-        cp_async_wait_all();
-        finish_ghosts(b0);
-        __syncthreads();
-    }
+    const int s_own = (x + 3) * kP + 4 + 2 * pr;            // this thread's pair
+    const int s_gap = (x + 3) * kP + kColY + pr;             // p+ of the row below it
+    // the row above an odd last row is the edge warps' (a halo row)
+    auto put_own = [&](T* b, L v) {
+        if (node1) put_lanes(b + s_own, v);
+        else if (node) b[s_own] = lane_a(v);
+    };
+    put_own(smem, q[2]);
+    if (D >= 3 && C.zbeg + 1 < C.zend) put_own(smem + buf, q[3]);
+    block_barrier(C.nt);
 
-    for (int z = zbeg; z < zend; ++z) {
-        const int fz = z * sS;
-        T* const bz = smem + ((z - zbeg) & 1) * buf_elems;        // plane z (and z+2)
-        T* const bn = smem + ((z - zbeg + 1) & 1) * buf_elems;    // plane z+1
-        T cosz = cos2, sinz = sin2;
-        if constexpr (D == 3 && uses_angle<D, DYN>()) {
-            cosz = trig[z];
-            sinz = trig_s[z];
-        }
-        if (D >= 3 && node)
-            q[5] = z_inside ? ld(ucol + fz + 3 * sS) : line_value(ucol, z + 3, ns, (long long)sS, perS, extrap);
-        T vv = T(0);
-        if constexpr (kVnAhead) {
-            if (node) {
-                vv = vn_next;
-                if (z + 1 < zend) vn_next = ld(vn + col + fz + sS);
+#pragma unroll 1
+    for (int z = C.zbeg; z < C.zend; ++z) {
+        T* const bz = smem + ((z - C.zbeg) & 1) * buf;
+        const T cosz = cos2, sinz = sin2;
+        T va = vn0, vb = vn1;
+        if constexpr (D >= 3) q[5] = q6;
+        // the next plane's values, a whole plane of work ahead of their use
+        if (D >= 3 && z + 1 < C.zend) {
+            if (z + 4 < ns) q6 = lanes(ld(u4 + f0), ld(u4 + f1));
+            else q6 = column(z + 4);
+            if constexpr (D == 3 && uses_angle<D, DYN>()) {
+                cos2 = trig[z + 1];
+                sin2 = trig_s[z + 1];
+            }
+            if constexpr (kVnAhead) {
+                vn0 = ld(vn_next + f0);
+                vn1 = ld(vn_next + f1);
             }
         }
 
         // phase A: interfaces of plane z along dimensions 0 and 1
-        T pmx = T(0), pmy = T(0);
-        // x-interface between nodes x-1 and x of row r (x = nx: the row's last one)
-        if (do_xrow) {
-            const T* a = bz + s_xrow;
-            T ppj;
-            iface_at<SCHEME>(a[0], a[1], a[2], a[3], a[4], a[5], fl0, ppj, pmx);
-            bz[s_pxp] = ppj;
-        }
-        // merged blocks: the last interface of row er (between node n0-1 and the ghost n0)
-        if (merged && spare) {
-            const T* a = bz + (er + 3) * W + nx;
-            T ppj, unused;
-            iface_at<SCHEME>(a[0], a[1], a[2], a[3], a[4], a[5], fl0, ppj, unused);
-            bz[o_pxp + er * (nx + 1) + nx] = ppj;
-        }
-        // y-interface of gap gk (between tile rows gk-1 and gk) of column x
-        if (gk >= 0) {
-            const T* c = bz + s_ycol;
-            T ppj;
-            iface_at<SCHEME>(c[0], c[W], c[2 * W], c[3 * W], c[4 * W], c[5 * W], fl1, ppj, pmy);
-            bz[s_pyw] = ppj;
-        }
-        if (do_ylast) {
-            const T* c = bz + s_ylast;
-            T ppj, unused;
-            iface_at<SCHEME>(c[0], c[W], c[2 * W], c[3 * W], c[4 * W], c[5 * W], fl1, ppj, unused);
-            bz[o_pyp + TY * nx + x] = ppj;
-        }
-        cp_async_wait_all();  // this thread's copies into plane z+1
-        if (z + 1 < zend) finish_ghosts(bn);
-        __syncthreads();
+        L pmx, pmy, pp;
+        const T* own = bz + s_own;
+        L w[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) w[k] = lanes_at(own + (k - 3) * kP);
+        iface_lanes<SCHEME>(w, fl0, pp, pmx);
+        if (node) put_lanes(bz + s_own + (kColX - 4), pp);
+        const L b2 = lanes_at(own - 4), b1 = lanes_at(own - 2), up = lanes_at(own + 2);
+        const T v[7] = {lane_b(b2), lane_a(b1), lane_b(b1), lane_a(w[3]), lane_b(w[3]), lane_a(up), lane_b(up)};
+        iface_line<SCHEME>(v, fl1, pp, pmy);
+        if (node) bz[s_gap] = lane_a(pp);
+        const T ppy_a = lane_b(pp);
+        block_barrier(C.nt);
 
-        // phase B: staging of plane z+2, then the node update of plane z
-        if (z + 2 < zend) {
-            if (node) bz[s_center] = q[4];
-            stage_rest(z + 2, bz);
+        // phase B: staging of plane z+2, then the node updates of plane z
+        const L ppx = lanes_at(bz + s_own + (kColX - 4) + kP);
+        const L ppy = lanes(ppy_a, bz[s_gap + 1]);
+        if (D >= 3 && z + 2 < C.zend) put_own(bz, q[4]);
+        // raw sums and differences of the one-sided derivatives
+        L sm[D], df[D];
+        sm[0] = pmx + ppx;
+        df[0] = ppx - pmx;
+        sm[1] = pmy + ppy;
+        df[1] = ppy - pmy;
+        if constexpr (D >= 3) {
+            L pps, next;
+            if constexpr (kSlide) {
+                za.slide(q[4].a, q[5].a);
+                za.eval(flS, pps.a, next.a);
+                zb.slide(q[4].b, q[5].b);
+                zb.eval(flS, pps.b, next.b);
+            } else {
+                iface_lanes<SCHEME>(q, flS, pps, next);
+            }
+            sm[SD] = carry + pps;
+            df[SD] = pps - carry;
+            carry = next;
         }
-        if (node) {
-            const T center = (D >= 3) ? q[2] : ld(ucol);
-            // raw sums and differences of the one-sided derivatives, and 1/(2 dx)
-            T sm[D], df[D], hh[D];
-            const T ppx = bz[s_pxp + 1];
-            const T ppy = bz[s_pyr];
-            sm[0] = pmx + ppx;
-            df[0] = ppx - pmx;
-            hh[0] = h0;
-            sm[1] = pmy + ppy;
-            df[1] = ppy - pmy;
-            hh[1] = h1;
-            T next = T(0);
-            if constexpr (D >= 3) {
-                T pps;
-                if constexpr (kSlide) {
-                    zline.slide(q[4], q[5]);
-                    zline.eval(flS, pps, next);
-                } else {
-                    iface_at<SCHEME>(q[0], q[1], q[2], q[3], q[4], q[5], flS, pps, next);
-                }
-                sm[SD] = carry + pps;
-                df[SD] = pps - carry;
-                hh[SD] = hS;
-            }
-            if constexpr (D == 4) {
-                // dimension 2: both interfaces of the node from a 7-point line
-                T v[7];
-                gather7<T>(u, (long long)(col + fz), i2, g.n[2], g.stride[2], (g.periodic_mask >> 2) & 1u, extrap, v);
-                T pm2, pp2, unused0, unused1;
-                const T fl2 = SP<T>::floor(P, 2);
-                iface_at<SCHEME>(v[0], v[1], v[2], v[3], v[4], v[5], fl2, unused0, pm2);
-                iface_at<SCHEME>(v[1], v[2], v[3], v[4], v[5], v[6], fl2, pp2, unused1);
-                sm[2] = pm2 + pp2;
-                df[2] = pp2 - pm2;
-                hh[2] = half_inv(2);
-                if constexpr (uses_coord<D, DYN>(3)) xc[3] = coord(SP<T>::lo(P, 3), z, SP<T>::dx(P, 3));
-            }
-            if constexpr (D == 3 && uses_coord<D, DYN>(2)) xc[2] = coord(SP<T>::lo(P, 2), z, SP<T>::dx(P, 2));
-            T yd = lf_combine_raw<T, D, DYN>(P, xc, cosz, sinz, sm, df, hh, alpha_global);
+        if constexpr (D == 4) {
+            // dimension 2: both interfaces of each node from a 7-point line
+            T v0[7], v1[7];
+            const bool per2 = (g.periodic_mask >> 2) & 1u;
+            gather7<T>(u, (long long)f0, C.i2, g.n[2], g.stride[2], per2, extrap, v0);
+            gather7<T>(u, (long long)f1, C.i2, g.n[2], g.stride[2], per2, extrap, v1);
+            L l[7], pm2, pp2, unused0, unused1;
+#pragma unroll
+            for (int k = 0; k < 7; ++k) l[k] = lanes(v0[k], v1[k]);
+            const T fl2 = SP<T>::floor(P, 2);
+            iface_lanes<SCHEME>(l, fl2, unused0, pm2);
+            iface_lanes<SCHEME>(l + 1, fl2, pp2, unused1);
+            sm[2] = pm2 + pp2;
+            df[2] = pp2 - pm2;
+            if constexpr (uses_coord<D, DYN>(3)) xa[3] = xb[3] = coord(SP<T>::lo(P, 3), z, SP<T>::dx(P, 3));
+        }
+        if constexpr (D == 3 && uses_coord<D, DYN>(2)) xa[2] = xb[2] = coord(SP<T>::lo(P, 2), z, SP<T>::dx(P, 2));
+        auto node_value = [&](const T* xc, const T* S, const T* Q, T center, T old) -> T {
+            T yd = lf_node<T, D, DYN>(P, xc, cosz, sinz, S, Q, hh, alpha_global);
+            // BRT min(0, .) as a clamp; FP64 on the bit pattern: positive values (and +NaN) become 0
             if constexpr (std::is_same<T, double>::value) {
-                // BRT min(0, .) on the bit pattern: positive values (and +NaN) become 0
                 if (brt0 && __double_as_longlong(yd) > 0) yd = 0.0;
             } else {
                 yd = fminf(yd, clamp);
             }
-            const int flat = col + fz;
+            if constexpr (KIND == kKindTerm) return yd;
+            const T w = fma_rn(dt, yd, center);
+            if constexpr (KIND != kKindCombine) return w;
+            // cv V^n + cu w; with cv + cu = 1 FP32 takes it as w + cv (V^n - w): the
+            // difference is small, so that one rounding alone counts
             T res;
-            if constexpr (KIND == kKindTerm) {
-                res = yd;
-            } else if constexpr (KIND == kKindFirst) {
-                res = center + dt * yd;
-            } else {
-                if constexpr (!kVnAhead) vv = ld(vn + flat);
-                res = cv * vv + cu * (center + dt * yd);
-                if (minv) res = fmin(res, vv);
-            }
-            out[flat] = res;
-            if (also_out) also_out[flat] = res;
-            if constexpr (D >= 3) {
-                carry = next;
+            if constexpr (std::is_same<T, double>::value) res = fma_rn(cu, w, mul_rn(cv, old));
+            else res = fma_rn(cv, add_rn(old, -w), w);
+            return minv ? fmin(res, old) : res;
+        };
+        if constexpr (KIND == kKindCombine && !kVnAhead) {
+            va = ld(vn + f0);
+            vb = ld(vn + f1);
+        }
+        T S[D], Q[D];
 #pragma unroll
-                for (int k = 0; k < 5; ++k) q[k] = q[k + 1];
-            }
+        for (int d = 0; d < D; ++d) { S[d] = lane_a(sm[d]); Q[d] = lane_a(df[d]); }
+        const T ra = node_value(xa, S, Q, lane_a(q[2]), va);
+#pragma unroll
+        for (int d = 0; d < D; ++d) { S[d] = lane_b(sm[d]); Q[d] = lane_b(df[d]); }
+        const T rb = node_value(xb, S, Q, lane_b(q[2]), vb);
+        if (node) out[f0] = ra;
+        if (node1) out[f1] = rb;
+        if (also_out) {
+            if (node) also_out[f0] = ra;
+            if (node1) also_out[f1] = rb;
+        }
+        f0 += sS;
+        f1 += sS;
+        if constexpr (D >= 3) {
+#pragma unroll
+            for (int k = 0; k < 5; ++k) q[k] = q[k + 1];
         }
     }
 }
 
-// Whether tile (row_tile, chunk) is interior: all its TY rows and three halo
-// rows on each side inside the grid along dimension 1, and its chunk's planes
-// with three on each side inside the grid along the streamed dimension.
-template <int D>
-__device__ __forceinline__ bool rows_interior(const GridDev& g, int ty, int tz, int row_tile, int chunk) {
-    const int y0 = row_tile * ty;
-    bool in = y0 >= 3 && y0 + ty + 3 <= g.n[1];
-    if constexpr (D >= 3) {
-        const int zbeg = chunk * tz, zend = min(g.n[D - 1], zbeg + tz);
-        in = in && zbeg >= 3 && zend + 3 <= g.n[D - 1];
-    }
-    return in;
+template <typename T, int D, int DYN, int SCHEME, int KIND>
+__device__ __forceinline__ void rows_tile(const StageParams& P, const StageRun<T>& R, const int SX, const int TY,
+                                          const int NT, const int tz, const int tile, const int i2, const int chunk,
+                                          const int t, T* const smem) {
+    const GridDev& g = P.g;
+    const int nseg = (g.n[0] + SX - 1) / SX;
+    const int row_tile = tile / nseg, seg = tile - row_tile * nseg;
+    constexpr int SD = (D >= 3) ? D - 1 : 0;
+    Tile C;
+    C.x0 = seg * SX;
+    C.sx = min(SX, g.n[0] - C.x0);
+    C.y0 = row_tile * TY;
+    C.rv = min(TY, g.n[1] - C.y0);
+    C.i2 = (D == 4) ? i2 : 0;
+    C.zbeg = (D >= 3) ? chunk * tz : 0;
+    C.zend = (D >= 3) ? min(g.n[SD], C.zbeg + tz) : 1;
+    C.stride = SX;
+    C.nn = rows_node_threads(SX, TY);
+    C.nt = NT;
+    const int buf = rows_buf_elems(SX);
+    if (t < C.nn) node_warps<T, D, DYN, SCHEME, KIND>(P, R, C, t, smem, buf);
+    else edge_warps<T, D, SCHEME>(P, R.u, C, t, smem, buf);
 }
 
-template <typename T, int D, int DYN, int SCHEME, int KIND, int OCC>
-__global__ void __launch_bounds__(RowsBounds<T, OCC>::kThreads, OCC) rows_kernel(const StageParams P, const RowsCfg C) {
+template <typename T, int D, int DYN, int SCHEME, int KIND>
+__global__ void __launch_bounds__(RowsLimits<T>::kThreads, 1) rows_kernel(const StageParams P, const RowsCfg C) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const StageRun<T> R = stage_run<T>(P);
     const int i2 = (D == 4) ? (int)blockIdx.y : 0;
     const int chunk = (D == 3) ? (int)blockIdx.y : ((D == 4) ? (int)blockIdx.z : 0);
-    // the interior body is compiled for the ENO schemes only: there it pays
-    // (their per-node arithmetic is small beside the staging logic), while a
-    // second WENO5 body measured slower in FP32 and no faster in FP64
-    if constexpr (SCHEME != HJ_WENO5) {
-        if (C.split && rows_interior<D>(P.g, C.ty, C.tz, blockIdx.x, chunk)) {
-            rows_tile<T, D, DYN, SCHEME, KIND, true>(P, R, C.ty, C.nt, C.tz, blockIdx.x, i2, chunk, threadIdx.x,
-                                                     reinterpret_cast<T*>(smem_raw));
-            return;
-        }
-    }
-    rows_tile<T, D, DYN, SCHEME, KIND, false>(P, R, C.ty, C.nt, C.tz, blockIdx.x, i2, chunk, threadIdx.x,
-                                              reinterpret_cast<T*>(smem_raw));
+    grid_wait();
+    rows_tile<T, D, DYN, SCHEME, KIND>(P, R, C.sx, C.ty, C.nt, C.tz, blockIdx.x, i2, chunk, threadIdx.x,
+                                       reinterpret_cast<T*>(smem_raw));
 }
 
-// Shared memory of a rows_kernel block.
-template <typename T>
-inline size_t rows_smem_bytes(int nx, int ty) {
-    return rows_smem(nx, ty, sizeof(T));
-}
-
-template <typename T, int D, int DYN>
-inline void rows_shape(const StageParams& p, const RowsCfg& c, dim3& grid, dim3& block, size_t& smem) {
+template <int D>
+inline void rows_shape(const StageParams& p, const RowsCfg& c, dim3& grid, dim3& block) {
     block = dim3((unsigned)c.nt, 1, 1);
-    grid = dim3((unsigned)c.row_tiles, 1, 1);
+    grid = dim3((unsigned)c.tiles, 1, 1);
     if (D == 3) grid.y = (unsigned)c.nchunks;
     if (D == 4) { grid.y = (unsigned)p.g.n[2]; grid.z = (unsigned)c.nchunks; }
-    smem = rows_smem_bytes<T>(p.g.n[0], c.ty);
 }
 
 // Opts a kernel into 200 KiB of dynamic shared memory, once per device (the
@@ -566,30 +541,19 @@ inline cudaError_t smem_optin(K* kernel, std::atomic<unsigned long long>& done) 
     return cudaSuccess;
 }
 
-template <typename T, int D, int DYN, int SCHEME, int KIND, int OCC>
+template <typename T, int D, int DYN, int SCHEME, int KIND>
 inline cudaError_t rows_prepare() {
     static std::atomic<unsigned long long> done{0};
-    return smem_optin(rows_kernel<T, D, DYN, SCHEME, KIND, OCC>, done);
+    return smem_optin(rows_kernel<T, D, DYN, SCHEME, KIND>, done);
 }
 
-template <typename T, int D, int DYN, int SCHEME, int KIND, int OCC>
-cudaError_t launch_rows_occ(const StageParams& p, const RowsCfg& c, cudaStream_t s) {
-    dim3 grid, block;
-    size_t smem;
-    rows_shape<T, D, DYN>(p, c, grid, block, smem);
-    cudaError_t e = rows_prepare<T, D, DYN, SCHEME, KIND, OCC>();
-    if (e != cudaSuccess) return e;
-    rows_kernel<T, D, DYN, SCHEME, KIND, OCC><<<grid, block, smem, s>>>(p, c);
-    return cudaGetLastError();
-}
-
-// The variant for two blocks per SM exists for FP32 only.
 template <typename T, int D, int DYN, int SCHEME, int KIND>
 cudaError_t launch_rows_kind(const StageParams& p, const RowsCfg& c, cudaStream_t s) {
-    if constexpr (std::is_same<T, float>::value) {
-        if (c.occ == 2) return launch_rows_occ<T, D, DYN, SCHEME, KIND, 2>(p, c, s);
-    }
-    return launch_rows_occ<T, D, DYN, SCHEME, KIND, 1>(p, c, s);
+    dim3 grid, block;
+    rows_shape<D>(p, c, grid, block);
+    cudaError_t e = rows_prepare<T, D, DYN, SCHEME, KIND>();
+    if (e != cudaSuccess) return e;
+    return launch_dependent(rows_kernel<T, D, DYN, SCHEME, KIND>, grid, block, rows_smem(c.sx, sizeof(T)), s, p, c);
 }
 
 template <typename T, int D, int DYN, int SCHEME>
@@ -617,28 +581,17 @@ cudaError_t launch_rows_eno3(const StageParams& p, const RowsCfg& c, cudaStream_
     return launch_rows_scheme<T, D, DYN, HJ_ENO3>(p, c, s);
 }
 
-template <typename T, int D, int DYN, int SCHEME, int OCC>
-int rows_bps_occ(const StageParams& p, const RowsCfg& c) {
-    dim3 grid, block;
-    size_t smem;
-    rows_shape<T, D, DYN>(p, c, grid, block, smem);
-    if ((int)block.x > RowsBounds<T, OCC>::kThreads) return 0;
-    if (rows_prepare<T, D, DYN, SCHEME, kKindCombine, OCC>() != cudaSuccess) return 0;
-    int bps = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, rows_kernel<T, D, DYN, SCHEME, kKindCombine, OCC>,
-                                                      (int)block.x, smem) != cudaSuccess)
-        return 0;
-    return bps;
-}
-
 // Resident blocks per SM of the stage kernels of a configuration (the
 // combining stages, the largest of the three kinds); 0 if it cannot launch.
 template <typename T, int D, int DYN, int SCHEME>
 int rows_bps_scheme(const StageParams& p, const RowsCfg& c) {
-    if constexpr (std::is_same<T, float>::value) {
-        if (c.occ == 2) return rows_bps_occ<T, D, DYN, SCHEME, 2>(p, c);
-    }
-    return rows_bps_occ<T, D, DYN, SCHEME, 1>(p, c);
+    if (c.nt > RowsLimits<T>::kThreads) return 0;
+    if (rows_prepare<T, D, DYN, SCHEME, kKindCombine>() != cudaSuccess) return 0;
+    int bps = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, rows_kernel<T, D, DYN, SCHEME, kKindCombine>, c.nt,
+                                                      rows_smem(c.sx, sizeof(T))) != cudaSuccess)
+        return 0;
+    return bps;
 }
 template <typename T, int D, int DYN>
 int rows_bps_weno5(const StageParams& p, const RowsCfg& c) {

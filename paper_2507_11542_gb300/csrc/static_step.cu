@@ -9,6 +9,7 @@
 // block and fragment, or a host application that owns the GPU's memory pool
 // and forbids any other allocator. This entry point lets them step a value
 // function in a buffer they already own.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -112,40 +113,27 @@ bool method_valid(const hj_grid* g, const hj_method* m) {
     }
 }
 
-// Launch shape of the row kernel without timing: the fewest rows per tile
-// that give at least 256 threads, and planes per chunk so that the blocks
-// fill the SMs about twice.
+// Launch shape of the row kernel without timing: tiles of at most 256 node
+// threads (128 in FP64), and planes per chunk so that the blocks fill the SMs
+// about twice.
 bool pick_rows(const StageParams& P, int dtype, int sm_count, RowsCfg* c) {
     const GridDev& G = P.g;
     const int D = G.ndim;
     if (!rows_supported(D, P.dynamics)) return false;
     for (int d = 0; d < D; ++d)
         if (G.n[d] < 4) return false;
-    const int max_threads = rows_max_threads(dtype == HJ_F64);
-    const int nx = G.n[0], ny = G.n[1];
-    if (nx + 1 > max_threads) return false;
-    int ty = 1;
-    while (ty < ny && (nx + 1) * (ty + 2) <= max_threads && (nx + 1) * ty < 256) ++ty;
-    const size_t es = dtype == HJ_F64 ? 8 : 4;
-    if (rows_smem(nx, ty, es) > 200 * 1024) return false;
-    c->ty = ty;
-    c->nt = rows_block_threads(nx, ty, max_threads);
-    c->occ = 1;
-    c->split = 1;  // interior tiles on the body without ghost logic (the same bits either way)
-    c->row_tiles = (ny + ty - 1) / ty;
+    if (G.n[0] + 1 > rows_max_nodes(dtype == HJ_F64)) return false;
+    const int ty = std::min(D == 2 ? 4 : kRowsMaxTy, G.n[1]);
+    const int sx = rows_segment(G.n[0], ty, dtype == HJ_F64 ? 128 : 256);
     const int ns = D >= 3 ? G.n[D - 1] : 1;
-    const long long per_plane = (long long)c->row_tiles * (D == 4 ? G.n[2] : 1);
-    int tz = ns;
+    *c = make_rows_cfg(G, sx, ty, ns, rows_node_threads(sx, ty) + rows_edge_threads(sx));
     if (D >= 3) {
-        const long long want = 2LL * sm_count;
-        const long long chunks = (want + per_plane - 1) / per_plane;
-        tz = (int)std::max(1LL, (ns + chunks - 1) / std::max(1LL, chunks));
+        const long long per_plane = (long long)c->tiles * (D == 4 ? G.n[2] : 1);
+        const long long chunks = (2LL * sm_count + per_plane - 1) / per_plane;
+        *c = make_rows_cfg(G, sx, ty, (int)std::max(1LL, (ns + chunks - 1) / std::max(1LL, chunks)), c->nt);
     }
-    c->tz = D >= 3 ? tz : 1;
-    c->nchunks = D >= 3 ? (ns + c->tz - 1) / c->tz : 1;
     if (c->nchunks > 65535) return false;
-    const int bps = dtype == HJ_F64 ? rows_blocks_per_sm_f64(P, *c) : rows_blocks_per_sm_f32(P, *c);
-    return bps > 0;
+    return (dtype == HJ_F64 ? rows_blocks_per_sm_f64(P, *c) : rows_blocks_per_sm_f32(P, *c)) > 0;
 }
 
 }  // namespace

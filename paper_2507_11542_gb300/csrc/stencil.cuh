@@ -10,16 +10,31 @@
 
 #include "../../include/hj.h"
 #include "hj_internal.h"
+#include "launch.cuh"
 #include "weno_iface.cuh"
 
 namespace hj {
 
-template <typename T> __device__ __forceinline__ T ld(const T* p) { return __ldg(p); }
+// A load from global memory that stays behind grid_wait() (launch.cuh): a
+// read-only (.nc) load may be moved above it, and read what the kernel before
+// this one has not written yet.
+__device__ __forceinline__ float ld(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ double ld(const double* p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
 
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
 // |x|, and the maximum of two non-negative values, for FP64 as integer
 // operations on the bit patterns (non-negative doubles order like their bits):
@@ -405,20 +420,89 @@ __device__ __forceinline__ T lf_combine(const StageParams& P, const T* xc, T c, 
     return y;
 }
 
-// The Lax-Friedrichs term from the raw (undivided) one-sided derivatives:
-// sums S_d = p-_d + p+_d and differences Q_d = p+_d - p-_d, with h_d =
-// 1/(2 dx_d), so that the mean is h_d S_d and the half difference h_d Q_d.
-// (Folding h_d into the air3D coefficients instead was measured slower.)
+// The Lax-Friedrichs term of a node from the raw (undivided) one-sided
+// derivatives: sums S_d = p-_d + p+_d and differences Q_d = p+_d - p-_d, with
+// h_d = 1/(2 dx_d), so that the mean is h_d S_d and the half difference h_d Q_d.
+// The same formulas as lf_combine, every operation rounded as written (none is
+// left to contraction, so that every kernel that holds this code rounds alike).
+// Scalar in FP32 too: most operations take a value that is the same for the
+// whole block, which a packed one would want in a register pair.
 template <typename T, int D, int DYN>
-__device__ __forceinline__ T lf_combine_raw(const StageParams& P, const T* xc, T c, T s, const T* S, const T* Q,
-                                            const T* h, bool alpha_global) {
-    T pb[D], dd[D];
+__device__ __forceinline__ T lf_node(const StageParams& P, const T* x, T c, T s, const T* S, const T* Q, const T* h,
+                                     bool alpha_global) {
+    const auto q = [&P](int k) { return SP<T>::param(P, k); };
+    constexpr int B = dyn_base(DYN);
+    T pb[D], dd[D], a[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-        pb[d] = S[d] * h[d];
-        dd[d] = Q[d] * h[d];
+        pb[d] = mul_rn(S[d], h[d]);
+        dd[d] = mul_rn(Q[d], h[d]);
+        a[d] = T(0);
     }
-    return lf_combine<T, D, DYN>(P, xc, c, s, pb, dd, alpha_global);
+    T y;
+    if constexpr (B == HJ_DYN_DOUBLE_INTEGRATOR && D == 2) {
+        y = fma_rn(-q(0), absv(pb[1]), mul_rn(pb[0], x[1]));
+        a[0] = absv(x[1]);
+        a[1] = q(0);
+    } else if constexpr (B == HJ_DYN_AIR3D && D == 3) {
+        const T amax = q(2), bmax = q(3);
+        const T f0 = fma_rn(q(1), c, -q(0)), f1 = mul_rn(q(1), s);
+        const T k = fma_rn(x[0], pb[1], fma_rn(-x[1], pb[0], pb[2]));  // its sign does not matter
+        y = fma_rn(pb[1], f1, mul_rn(pb[0], f0));
+        y = fma_rn(-bmax, absv(pb[2]), fma_rn(amax, absv(k), y));
+        a[0] = fma_rn(amax, absv(x[1]), absv(f0));
+        a[1] = fma_rn(amax, absv(x[0]), absv(f1));
+        a[2] = add_rn(amax, bmax);
+    } else if constexpr (B == HJ_DYN_ROCKETS && D == 3) {
+        const T ac = q(0), g = q(1), ue = q(2), up = q(3);
+        const T f0 = mul_rn(ac, c), f1 = add_rn(fma_rn(ac, s, ac), -g);
+        const T ke = fma_rn(-x[0], pb[0], pb[2]), kp = fma_rn(x[0], pb[1], pb[2]);
+        y = fma_rn(pb[1], f1, mul_rn(pb[0], f0));
+        y = fma_rn(-up, absv(kp), fma_rn(ue, absv(ke), y));
+        a[0] = fma_rn(ue, absv(x[0]), absv(f0));
+        a[1] = fma_rn(up, absv(x[0]), absv(f1));
+        a[2] = add_rn(ue, up);
+    } else if constexpr (B == HJ_DYN_DUBINS4D && D == 4) {
+        const T wmax = q(0), accmax = q(1);
+        const T f0 = mul_rn(x[3], c), f1 = mul_rn(x[3], s);
+        y = fma_rn(pb[1], f1, mul_rn(pb[0], f0));
+        y = fma_rn(-accmax, absv(pb[3]), fma_rn(-wmax, absv(pb[2]), y));
+        a[0] = absv(f0);
+        a[1] = absv(f1);
+        a[2] = wmax;
+        a[3] = accmax;
+    } else if constexpr (B == HJ_DYN_NORM) {
+        T s2 = mul_rn(pb[0], pb[0]);
+        a[0] = q(0);
+#pragma unroll
+        for (int d = 1; d < D; ++d) {
+            s2 = fma_rn(pb[d], pb[d], s2);
+            a[d] = q(0);
+        }
+        y = mul_rn(-q(0), sqrt(s2));
+    } else if constexpr (B == HJ_DYN_ADVECT) {
+        y = mul_rn(-q(0), pb[0]);
+        a[0] = absv(q(0));
+#pragma unroll
+        for (int d = 1; d < D; ++d) {
+            y = fma_rn(-q(d), pb[d], y);
+            a[d] = absv(q(d));
+        }
+    } else {
+        static_assert(B == HJ_DYN_ROTATE && D >= 2, "a dynamics of the row kernel");
+        const T f0 = mul_rn(q(0), x[1]), f1 = mul_rn(q(0), x[0]);  // the speeds are -f0, f1
+        y = fma_rn(-f1, pb[1], mul_rn(f0, pb[0]));
+        a[0] = absv(f0);
+        a[1] = absv(f1);
+    }
+    if constexpr (dyn_is_box(DYN)) box_alpha<T, D, B>(P, x, c, s, pb, dd, a);
+    if (alpha_global) {
+#pragma unroll
+        for (int d = 0; d < D; ++d) a[d] = SP<T>::alpha_g(P, d);
+    }
+#pragma unroll
+    for (int d = 0; d < D; ++d) y = fma_rn(a[d], dd[d], y);
+    return y;
 }
 
 // Whether a dynamics reads the coordinate of dimension d (the others are not computed).

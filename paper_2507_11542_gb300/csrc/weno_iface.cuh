@@ -30,6 +30,8 @@
 #include <type_traits>
 
 #include "../../include/hj.h"
+#include "hj_internal.h"
+#include "lanes.cuh"
 #include "weno_weights64.cuh"
 
 namespace hj {
@@ -40,40 +42,53 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return r;
 }
 
-// FP32, rescaled in ways that leave every weight unchanged: smoothness values
-// and epsilon times 4 (S' = 13/3 t^2 + u^2), ideal weights times 10; results
-// times 6 (the caller divides the 6 out with 1/(2 dx)); with one reciprocal per weight and per
-// side: (S' + eps')^2 >= (4e-18)^2 stays a normal number, so the approximate
-// reciprocals neither overflow nor divide by zero. No a*b + c is left for the
-// compiler to contract, so every inlined copy rounds alike.
-__device__ __forceinline__ void weno_iface(float e1, float e2, float e3, float e4, float e5, float floor_raw,
-                                           float& pp_j, float& pm_j1) {
-    const float tA = fmaf(-2.0f, e2, e1) + e3;
-    const float tB = fmaf(-2.0f, e3, e2) + e4;
-    const float tC = fmaf(-2.0f, e4, e3) + e5;
-    const float uA = fmaf(2.0f, e3 - e2, tA);  // e1 - 4e2 + 3e3
-    const float uB = e2 - e4;
-    const float uC = fmaf(2.0f, e3 - e4, tC);  // 3e3 - 4e4 + e5
-    const float SA = fmaf(uA, uA, (13.0f / 3.0f * tA) * tA);
-    const float SB = fmaf(uB, uB, (13.0f / 3.0f * tB) * tB);
-    const float SC = fmaf(uC, uC, (13.0f / 3.0f * tC) * tC);
-    const float amax = fmaxf(fmaxf(fmaxf(fabsf(e1), fabsf(e2)), fmaxf(fabsf(e3), fabsf(e4))), fabsf(e5));
-    const float eps = fmaf(4e-6f, amax * amax, 4.0f * floor_raw);
-    const float sA = SA + eps, sB = SB + eps, sC = SC + eps;
-    const float rA = rcp_approx(sA * sA);
-    const float rB = rcp_approx(sB * sB);
-    const float rC = rcp_approx(sC * sC);
-    const float T1 = tA - tB, T2 = tB - tC;
-    const float X = rA * T1, Y = rC * T2;
-    const float XY = __fadd_rn(X, Y);
-    const float numL = fmaf(2.0f, XY, Y);  // 2X + 3Y
-    const float numR = fmaf(2.0f, XY, X);  // 3X + 2Y
-    const float DL = fmaf(3.0f, rC, fmaf(6.0f, rB, rA));
-    const float DR = fmaf(3.0f, rA, fmaf(6.0f, rB, rC));
-    const float phi6 = fmaf(5.0f, e3, fmaf(2.0f, e4, -e2));  // 6 phi2
-    const float psi6 = fmaf(3.0f, uB, phi6);                 // 6 psi2
-    pm_j1 = fmaf(numL, rcp_approx(DL), phi6);
-    pp_j = fmaf(-numR, rcp_approx(DR), psi6);
+// FP32, two interfaces at a time (one per lane), rescaled in ways that leave
+// every weight unchanged: smoothness values and epsilon times 4 (S' = 13/3 t^2
+// + u^2), ideal weights times 10; results times 6 (the caller divides the 6 out
+// with 1/(2 dx)), written around the interface's own difference as in FP64
+// below. One reciprocal per weight and per side: (S' + eps')^2 >= (4e-18)^2
+// stays a normal number, so the approximate reciprocals neither overflow nor
+// divide by zero.
+//
+// The FP32 kernels are bound by instruction issue: 42 packed instructions, 10
+// reciprocals and 12 scalar ones for both interfaces, where one alone took 57
+// and 5 reciprocals with scalar instructions. A packed constant is a register
+// pair, so the formulas get by with three (2, 6, 13/3), and use sums where they
+// can: with m = e2 - e4 = -(d23 + d34), 2 d34 + d23 = d34 - m and -(2 d23 + d34)
+// = m - d23; squares take either sign. No product's only use is a sum: packed
+// products and sums are contracted too, and each inlined copy has to round
+// alike.
+__device__ __forceinline__ float eps_of(float e1, float e2, float e3, float e4, float e5) {
+    const float a = fmaxf(fmaxf(fabsf(e1), fabsf(e2)), fabsf(e3));
+    const float amax = fmaxf(fmaxf(a, fabsf(e4)), fabsf(e5));
+    return __fmaf_rn(__fmul_rn(4e-6f, amax), amax, 4.0f * kWenoFloorF32);
+}
+__device__ __forceinline__ F2 rcp2(F2 x) { return lanes(rcp_approx(lane_a(x)), rcp_approx(lane_b(x))); }
+
+__device__ __forceinline__ void weno_iface2(F2 e1, F2 e2, F2 e3, F2 e4, F2 e5, F2& pp_j, F2& pm_j1) {
+    const F2 two = both(2.0f), six = both(6.0f), c133 = both(13.0f / 3.0f);
+    const F2 d12 = e2 - e1, d23 = e3 - e2, d34 = e4 - e3, d45 = e5 - e4;
+    const F2 tA = d23 - d12, tB = d34 - d23, nC = d34 - d45;  // nC = -tC
+    const F2 uA = fma2(two, d23, tA);  // e1 - 4e2 + 3e3
+    const F2 m = e2 - e4;
+    const F2 uC = fma2(two, d34, nC);  // -(3e3 - 4e4 + e5)
+    const F2 eps = lanes(eps_of(lane_a(e1), lane_a(e2), lane_a(e3), lane_a(e4), lane_a(e5)),
+                         eps_of(lane_b(e1), lane_b(e2), lane_b(e3), lane_b(e4), lane_b(e5)));
+    const F2 sA = fma2(uA, uA, fma2(c133 * tA, tA, eps));
+    const F2 sB = fma2(m, m, fma2(c133 * tB, tB, eps));
+    const F2 sC = fma2(uC, uC, fma2(c133 * nC, nC, eps));
+    const F2 rA = rcp2(sA * sA), rB = rcp2(sB * sB), rC = rcp2(sC * sC);
+    const F2 T1 = tA - tB, T2 = tB + nC;
+    const F2 X = rA * T1, Y = rC * T2;
+    const F2 XY = fma2(rA, T1, Y);
+    const F2 numL = fma2(two, XY, Y);  // 2X + 3Y
+    const F2 numR = fma2(two, XY, X);  // 3X + 2Y
+    const F2 all = fma2(six, rB, rA + rC);
+    const F2 DL = fma2(two, rC, all), DR = fma2(two, rA, all);
+    const F2 sL = fma2(numL, rcp2(DL), d34 - m);
+    const F2 sR = fma2(numR, neg2(rcp2(DR)), m - d23);
+    pm_j1 = fma2(six, e3, sL);
+    pp_j = fma2(six, e3, sR);
 }
 
 // 1/x for a positive normal double: the hardware estimate refined by two
@@ -226,19 +241,70 @@ __device__ __forceinline__ void eno3_iface(T v0, T v1, T v2, T v3, T v4, T v5, T
     pm_j1 = e2 + T(0.5) * c + (left ? T(2) * third : -third);
 }
 
-// The interface between nodes j and j+1 from the values at nodes j-2 .. j+3
-// (WENO5 and ENO3 read all six, ENO2 the middle four, ENO1 the middle two:
-// first order takes the difference across the interface for both sides).
-template <int SCHEME, typename T>
-__device__ __forceinline__ void iface_at(T v0, T v1, T v2, T v3, T v4, T v5, T floor_raw, T& pp_j, T& pm_j1) {
-    if constexpr (SCHEME == HJ_ENO1) {
-        pp_j = pm_j1 = v3 - v2;
-    } else if constexpr (SCHEME == HJ_ENO2) {
-        eno2_iface(v1, v2, v3, v4, pp_j, pm_j1);
-    } else if constexpr (SCHEME == HJ_ENO3) {
-        eno3_iface(v0, v1, v2, v3, v4, v5, pp_j, pm_j1);
+// Two interfaces at a time, one per lane: w0..w5 hold the values at the nodes
+// j-2 .. j+3 of each (WENO5 and ENO3 read all six, ENO2 the middle four, ENO1
+// the middle two: first order takes the difference across the interface for
+// both sides).
+template <int SCHEME>
+__device__ __forceinline__ void iface_lanes(const F2 w[6], float, F2& pp, F2& pm) {
+    if constexpr (SCHEME == HJ_WENO5) {
+        weno_iface2(w[1] - w[0], w[2] - w[1], w[3] - w[2], w[4] - w[3], w[5] - w[4], pp, pm);
+    } else if constexpr (SCHEME == HJ_ENO1) {
+        pp = pm = w[3] - w[2];
     } else {
-        weno_iface(v1 - v0, v2 - v1, v3 - v2, v4 - v3, v5 - v4, floor_raw, pp_j, pm_j1);
+        float pa, pb, ma, mb;
+        if constexpr (SCHEME == HJ_ENO2) {
+            eno2_iface(lane_a(w[1]), lane_a(w[2]), lane_a(w[3]), lane_a(w[4]), pa, ma);
+            eno2_iface(lane_b(w[1]), lane_b(w[2]), lane_b(w[3]), lane_b(w[4]), pb, mb);
+        } else {
+            eno3_iface(lane_a(w[0]), lane_a(w[1]), lane_a(w[2]), lane_a(w[3]), lane_a(w[4]), lane_a(w[5]), pa, ma);
+            eno3_iface(lane_b(w[0]), lane_b(w[1]), lane_b(w[2]), lane_b(w[3]), lane_b(w[4]), lane_b(w[5]), pb, mb);
+        }
+        pp = lanes(pa, pb);
+        pm = lanes(ma, mb);
+    }
+}
+template <int SCHEME>
+__device__ __forceinline__ void iface_lanes(const D2 w[6], double floor12, D2& pp, D2& pm) {
+    if constexpr (SCHEME == HJ_WENO5) {
+        weno_iface(w[1].a - w[0].a, w[2].a - w[1].a, w[3].a - w[2].a, w[4].a - w[3].a, w[5].a - w[4].a, floor12, pp.a,
+                   pm.a);
+        weno_iface(w[1].b - w[0].b, w[2].b - w[1].b, w[3].b - w[2].b, w[4].b - w[3].b, w[5].b - w[4].b, floor12, pp.b,
+                   pm.b);
+    } else if constexpr (SCHEME == HJ_ENO1) {
+        pp = pm = w[3] - w[2];
+    } else if constexpr (SCHEME == HJ_ENO2) {
+        eno2_iface(w[1].a, w[2].a, w[3].a, w[4].a, pp.a, pm.a);
+        eno2_iface(w[1].b, w[2].b, w[3].b, w[4].b, pp.b, pm.b);
+    } else {
+        eno3_iface(w[0].a, w[1].a, w[2].a, w[3].a, w[4].a, w[5].a, pp.a, pm.a);
+        eno3_iface(w[0].b, w[1].b, w[2].b, w[3].b, w[4].b, w[5].b, pp.b, pm.b);
+    }
+}
+
+// Two consecutive interfaces along a line from its seven values v0..v6 (lane a:
+// the interface v0..v5, lane b: v1..v6); FP64 WENO5 shares their differences
+// (9 of 14 each), with the same results bit for bit.
+template <int SCHEME>
+__device__ __forceinline__ void iface_line(const float v[7], float floor, F2& pp, F2& pm) {
+    F2 w[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) w[k] = lanes(v[k], v[k + 1]);
+    iface_lanes<SCHEME>(w, floor, pp, pm);
+}
+template <int SCHEME>
+__device__ __forceinline__ void iface_line(const double v[7], double floor12, D2& pp, D2& pm) {
+    if constexpr (SCHEME == HJ_WENO5) {
+        Weno5Line line;
+        line.start(v[0], v[1], v[2], v[3], v[4], v[5]);
+        line.eval(floor12, pp.a, pm.a);
+        line.slide(v[5], v[6]);
+        line.eval(floor12, pp.b, pm.b);
+    } else {
+        D2 w[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) w[k] = lanes(v[k], v[k + 1]);
+        iface_lanes<SCHEME>(w, floor12, pp, pm);
     }
 }
 
