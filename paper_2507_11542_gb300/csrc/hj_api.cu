@@ -367,6 +367,14 @@ std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtyp
               [](const std::pair<double, RowsCfg>& a, const std::pair<double, RowsCfg>& b) { return a.first < b.first; });
     std::vector<RowsCfg> out;
     for (size_t k = 0; k < scored.size() && k < 20; ++k) out.push_back(scored[k].second);
+    if (D == 2) {
+        // FP64 stages: 51^2 4.7 us with 7 x 6 nodes, 101^2 6.2 with 5 x 12, 201^2 9.2 with 16 x 9, 301^2 17.2
+        // with 16 x 8, 511^2 44 (the row kernel 11.4, 13.8, 19.1, 50 from 101^2 on); FP32 takes 2.5 to 2.8 us
+        // with either kernel up to 301^2
+        static const int shapes[][2] = {{5, 8},  {5, 12}, {7, 4},  {7, 6},  {8, 5},   {8, 8},
+                                        {12, 6}, {16, 8}, {16, 9}, {12, 12}, {16, 10}, {32, 8}};
+        for (const auto& sh : shapes) out.push_back(make_plane_cfg(G, std::min(sh[0], nx), std::min(sh[1], ny), f64));
+    }
     return out;
 }
 

@@ -41,10 +41,10 @@ struct NvtxRange {
 // this many nodes a block.
 inline int rows_max_nodes(int dtype_is_f64) { return dtype_is_f64 ? 512 : 1024; }
 // Largest block of the row-tiled kernels, and the share its node threads may
-// take (two nodes a thread; at least one warp is left for the tile's edges):
-// FP32 blocks of 896 threads may use 72 registers a thread, FP64 blocks of 384
-// threads 168.
-constexpr int kRowsThreadsF32 = 896, kRowsThreadsF64 = 384;
+// take (two nodes a thread; at least one warp is left for the tile's edges).
+// FP64 blocks of 384 threads may use 168 registers a thread; what FP32 may use
+// is RowsBounds (rows_kernel.cuh).
+constexpr int kRowsThreadsF32 = 640, kRowsThreadsF64 = 384;
 inline int rows_max_threads(int dtype_is_f64) { return dtype_is_f64 ? kRowsThreadsF64 : kRowsThreadsF32; }
 inline int rows_max_node_threads(int dtype_is_f64) { return dtype_is_f64 ? 256 : 512; }
 
@@ -154,6 +154,7 @@ struct RowsCfg {
     int tz;       // planes per chunk along the streamed (last) dimension
     int nchunks;  // chunks along the streamed dimension
     int tiles;    // ceil(n0 / sx) * ceil(n1 / ty)
+    int plane;    // 1: the kernel of one interface a thread (2-D grids, plane_kernel.cuh)
 };
 // threads of the node warps (two rows each)
 __host__ __device__ inline int rows_node_threads(int sx, int ty) { return (sx * ((ty + 1) / 2) + 31) / 32 * 32; }
@@ -180,7 +181,23 @@ inline RowsCfg make_rows_cfg(const GridDev& G, int sx, int ty, int tz, int nt) {
     const int ns = G.ndim >= 3 ? G.n[G.ndim - 1] : 1;
     c.tz = G.ndim >= 3 ? tz : 1;
     c.nchunks = (ns + c.tz - 1) / c.tz;
+    c.plane = 0;
     return c;
+}
+
+// The plane kernel's block: threads for the items of a tile (FP32: pairs of
+// interfaces), at most kPlaneThreads; and its shared memory.
+constexpr int kPlaneThreads = 384;
+inline RowsCfg make_plane_cfg(const GridDev& G, int sx, int ty, int dtype_is_f64) {
+    const int w = dtype_is_f64 ? 1 : 2;
+    const int items = (sx + 1) * ((ty + w - 1) / w) + sx * ((ty + w) / w);
+    const int nt = (items + 31) / 32 * 32;
+    RowsCfg c = make_rows_cfg(G, sx, ty, 1, nt < kPlaneThreads ? nt : kPlaneThreads);
+    c.plane = 1;
+    return c;
+}
+inline size_t plane_smem(int sx, int ty, size_t es) {
+    return es * ((size_t)(ty + 8) * (sx + 6) + 2 * (size_t)(ty + 1) * (sx + 1) + 2 * (size_t)(ty + 2) * sx);
 }
 
 // Launchers (one translation unit per element type). Return the launch error.

@@ -33,9 +33,12 @@
 
 namespace hj {
 
-template <typename T> struct RowsLimits;
-template <> struct RowsLimits<float> { static constexpr int kThreads = kRowsThreadsF32; };
-template <> struct RowsLimits<double> { static constexpr int kThreads = kRowsThreadsF64; };
+// Launch bounds, i.e. registers a thread (blocks have at most rows_max_threads).
+// FP32 stage of 101^3 / 161x113x79 at 640, 768, 896, 1024 threads (96, 80, 72, 64
+// registers): 16.7, 16.1, 15.7, 16.2 / 22.6, 20.5, 20.0, 20.7 us; of 81^4 at 768 and
+// 896: 0.69 and 0.71 ms.
+template <typename T, int D> struct RowsBounds { static constexpr int kThreads = D == 3 ? 896 : 768; };
+template <int D> struct RowsBounds<double, D> { static constexpr int kThreads = kRowsThreadsF64; };
 
 // The slope that ghost values continue outward, and the m-th ghost value.
 template <typename T>
@@ -72,6 +75,29 @@ __device__ __forceinline__ StageRun<T> stage_run(const StageParams& P) {
     R.minv = P.minv_after;
     R.brt0 = P.brt_min0;
     return R;
+}
+
+// What a stage stores at a node, from the raw sums and differences of its
+// one-sided derivatives (lf_node), its stage input `center` and its V^n `old`.
+template <typename T, int D, int DYN, int KIND>
+__device__ __forceinline__ T stage_value(const StageParams& P, const StageRun<T>& R, const T* par, const T* x, T c, T s,
+                                         const T* S, const T* Q, const T* h, bool alpha_global, T center, T old) {
+    T yd = lf_node<T, D, DYN>(P, par, x, c, s, S, Q, h, alpha_global);
+    // BRT min(0, .) as a clamp (+inf: none); FP64 on the bit pattern: positive values (and +NaN) become 0
+    if constexpr (std::is_same<T, double>::value) {
+        if (R.brt0 && __double_as_longlong(yd) > 0) yd = 0.0;
+    } else {
+        yd = fminf(yd, R.brt0 ? 0.0f : INFINITY);
+    }
+    if constexpr (KIND == kKindTerm) return yd;
+    const T w = fma_rn(R.dt, yd, center);
+    if constexpr (KIND != kKindCombine) return w;
+    // cv V^n + cu w; with cv + cu = 1 FP32 takes it as w + cv (V^n - w): the
+    // difference is small, so that one rounding alone counts
+    T res;
+    if constexpr (std::is_same<T, double>::value) res = fma_rn(R.cu, w, mul_rn(R.cv, old));
+    else res = fma_rn(R.cv, add_rn(old, -w), w);
+    return R.minv ? fmin(res, old) : res;
 }
 
 // Asynchronous copy of one element from global to shared memory (cp.async:
@@ -284,9 +310,10 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
     T hh[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) hh[d] = half_inv(d);
-    const T dt = R.dt, cv = R.cv, cu = R.cu;
-    const bool minv = R.minv, brt0 = R.brt0;
-    const T clamp = brt0 ? T(0) : T(INFINITY);  // BRT min(0, .) as a clamp (+inf: none)
+    // read before the loop: a batch's descriptors lie in global memory, which its stores may alias
+    T par[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) par[k] = SP<T>::param(P, k);
     const bool alpha_global = P.alpha_global;
     // node coordinates that do not change along the streamed dimension
     T xa[D], xb[D];
@@ -438,24 +465,6 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
             if constexpr (uses_coord<D, DYN>(3)) xa[3] = xb[3] = coord(SP<T>::lo(P, 3), z, SP<T>::dx(P, 3));
         }
         if constexpr (D == 3 && uses_coord<D, DYN>(2)) xa[2] = xb[2] = coord(SP<T>::lo(P, 2), z, SP<T>::dx(P, 2));
-        auto node_value = [&](const T* xc, const T* S, const T* Q, T center, T old) -> T {
-            T yd = lf_node<T, D, DYN>(P, xc, cosz, sinz, S, Q, hh, alpha_global);
-            // BRT min(0, .) as a clamp; FP64 on the bit pattern: positive values (and +NaN) become 0
-            if constexpr (std::is_same<T, double>::value) {
-                if (brt0 && __double_as_longlong(yd) > 0) yd = 0.0;
-            } else {
-                yd = fminf(yd, clamp);
-            }
-            if constexpr (KIND == kKindTerm) return yd;
-            const T w = fma_rn(dt, yd, center);
-            if constexpr (KIND != kKindCombine) return w;
-            // cv V^n + cu w; with cv + cu = 1 FP32 takes it as w + cv (V^n - w): the
-            // difference is small, so that one rounding alone counts
-            T res;
-            if constexpr (std::is_same<T, double>::value) res = fma_rn(cu, w, mul_rn(cv, old));
-            else res = fma_rn(cv, add_rn(old, -w), w);
-            return minv ? fmin(res, old) : res;
-        };
         if constexpr (KIND == kKindCombine && !kVnAhead) {
             va = ld(vn + f0);
             vb = ld(vn + f1);
@@ -463,10 +472,10 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
         T S[D], Q[D];
 #pragma unroll
         for (int d = 0; d < D; ++d) { S[d] = lane_a(sm[d]); Q[d] = lane_a(df[d]); }
-        const T ra = node_value(xa, S, Q, lane_a(q[2]), va);
+        const T ra = stage_value<T, D, DYN, KIND>(P, R, par, xa, cosz, sinz, S, Q, hh, alpha_global, lane_a(q[2]), va);
 #pragma unroll
         for (int d = 0; d < D; ++d) { S[d] = lane_b(sm[d]); Q[d] = lane_b(df[d]); }
-        const T rb = node_value(xb, S, Q, lane_b(q[2]), vb);
+        const T rb = stage_value<T, D, DYN, KIND>(P, R, par, xb, cosz, sinz, S, Q, hh, alpha_global, lane_b(q[2]), vb);
         if (node) out[f0] = ra;
         if (node1) out[f1] = rb;
         if (also_out) {
@@ -507,7 +516,7 @@ __device__ __forceinline__ void rows_tile(const StageParams& P, const StageRun<T
 }
 
 template <typename T, int D, int DYN, int SCHEME, int KIND>
-__global__ void __launch_bounds__(RowsLimits<T>::kThreads, 1) rows_kernel(const StageParams P, const RowsCfg C) {
+__global__ void __launch_bounds__(RowsBounds<T, D>::kThreads, 1) rows_kernel(const StageParams P, const RowsCfg C) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const StageRun<T> R = stage_run<T>(P);
     const int i2 = (D == 4) ? (int)blockIdx.y : 0;
@@ -547,8 +556,15 @@ inline cudaError_t rows_prepare() {
     return smem_optin(rows_kernel<T, D, DYN, SCHEME, KIND>, done);
 }
 
+// (plane_kernel.cuh)
+template <typename T, int DYN, int SCHEME, int KIND>
+cudaError_t launch_plane(const StageParams& p, const RowsCfg& c, cudaStream_t s);
+
 template <typename T, int D, int DYN, int SCHEME, int KIND>
 cudaError_t launch_rows_kind(const StageParams& p, const RowsCfg& c, cudaStream_t s) {
+    if constexpr (D == 2) {
+        if (c.plane) return launch_plane<T, DYN, SCHEME, KIND>(p, c, s);
+    }
     dim3 grid, block;
     rows_shape<D>(p, c, grid, block);
     cudaError_t e = rows_prepare<T, D, DYN, SCHEME, KIND>();
@@ -585,7 +601,8 @@ cudaError_t launch_rows_eno3(const StageParams& p, const RowsCfg& c, cudaStream_
 // combining stages, the largest of the three kinds); 0 if it cannot launch.
 template <typename T, int D, int DYN, int SCHEME>
 int rows_bps_scheme(const StageParams& p, const RowsCfg& c) {
-    if (c.nt > RowsLimits<T>::kThreads) return 0;
+    if (c.plane) return D == 2 && c.nt <= kPlaneThreads && plane_smem(c.sx, c.ty, sizeof(T)) <= 200 * 1024 ? 1 : 0;
+    if (c.nt > RowsBounds<T, D>::kThreads) return 0;
     if (rows_prepare<T, D, DYN, SCHEME, kKindCombine>() != cudaSuccess) return 0;
     int bps = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, rows_kernel<T, D, DYN, SCHEME, kKindCombine>, c.nt,
@@ -639,3 +656,5 @@ int rows_bps_eno3(const StageParams& p, const RowsCfg& c) {
 
 
 }  // namespace hj
+
+#include "plane_kernel.cuh"

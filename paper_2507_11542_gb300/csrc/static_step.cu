@@ -123,6 +123,11 @@ bool pick_rows(const StageParams& P, int dtype, int sm_count, RowsCfg* c) {
     for (int d = 0; d < D; ++d)
         if (G.n[d] < 4) return false;
     if (G.n[0] + 1 > rows_max_nodes(dtype == HJ_F64)) return false;
+    if (D == 2 && dtype == HJ_F64) {  // 101^2: 6.2 us a stage, the row kernel 11.4; 511^2: 44 and 50
+        *c = G.total < 15000 ? make_plane_cfg(G, std::min(5, G.n[0]), std::min(12, G.n[1]), 1)
+                             : make_plane_cfg(G, std::min(16, G.n[0]), std::min(8, G.n[1]), 1);
+        return true;
+    }
     const int ty = std::min(D == 2 ? 4 : kRowsMaxTy, G.n[1]);
     const int sx = rows_segment(G.n[0], ty, dtype == HJ_F64 ? 128 : 256);
     const int ns = D >= 3 ? G.n[D - 1] : 1;

@@ -428,9 +428,9 @@ __device__ __forceinline__ T lf_combine(const StageParams& P, const T* xc, T c, 
 // Scalar in FP32 too: most operations take a value that is the same for the
 // whole block, which a packed one would want in a register pair.
 template <typename T, int D, int DYN>
-__device__ __forceinline__ T lf_node(const StageParams& P, const T* x, T c, T s, const T* S, const T* Q, const T* h,
-                                     bool alpha_global) {
-    const auto q = [&P](int k) { return SP<T>::param(P, k); };
+__device__ __forceinline__ T lf_node(const StageParams& P, const T* par, const T* x, T c, T s, const T* S, const T* Q,
+                                     const T* h, bool alpha_global) {
+    const auto q = [par](int k) { return par[k]; };  // the dynamics' parameters, read once per thread
     constexpr int B = dyn_base(DYN);
     T pb[D], dd[D], a[D];
 #pragma unroll
