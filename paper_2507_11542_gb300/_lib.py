@@ -102,11 +102,13 @@ _vp = ctypes.c_void_p
 def load():
     """Load libhj.so; raises if it is missing (no CPU or eager fallback exists)."""
     global _lib
+    if _lib is not None:  # every entry point comes through here
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
                 raise RuntimeError("libhj.so is not built at %s; run paper_2507_11542_gb300.build.build()" % LIB_PATH)
-            L = ctypes.CDLL(LIB_PATH)
+            L = ctypes.CDLL(LIB_PATH)  # published below, once every prototype is set
             L.hj_ctx_create.argtypes = [ctypes.c_int32, _vp, _P(_vp)]
             L.hj_ctx_destroy.argtypes = [_vp]
             L.hj_ctx_destroy.restype = None

@@ -52,8 +52,8 @@ def _check_tensor(t, spec, name):
     import torch
     if not isinstance(t, torch.Tensor) or not t.is_cuda or not t.is_contiguous():
         raise ValueError("%s must be a contiguous CUDA tensor" % name)
-    if t.numel() != int(np.prod(spec.n)):
-        raise ValueError("%s has %d elements, the grid %d" % (name, t.numel(), int(np.prod(spec.n))))
+    if t.numel() != math.prod(spec.n):
+        raise ValueError("%s has %d elements, the grid %d" % (name, t.numel(), math.prod(spec.n)))
 
 
 def upwind(ctx: Context, spec, m: L.hj_method, V, dim: int):
