@@ -54,27 +54,107 @@ __global__ void __launch_bounds__(kBX * kBY) stage_kernel(const StageParams P) {
     }
 }
 
-template <typename T, int D, int SCHEME>
-__global__ void __launch_bounds__(kBX * kBY) upwind_kernel(const UpwindParams P) {
-    const GridDev& g = P.g;
-    const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i1 = (D > 1) ? (int)(blockIdx.y * blockDim.y + threadIdx.y) : 0;
-    if (i0 >= g.n[0] || (D > 1 && i1 >= g.n[1])) return;
-    const int nz = (D > 2 ? g.n[2] : 1) * (D > 3 ? g.n[3] : 1);
+// p- and p+ along one dimension, from one interface evaluation for the two nodes
+// it separates: interface j (0 .. n of a line of n nodes) gives p- of node j and
+// p+ of node j-1, so that no thread needs another's result. A thread walks over
+// a run of interfaces of one line (FP32: of two lines, one per lane), which in
+// FP64 WENO5 reuse their differences (Weno5Line: 15 FP64 instructions an
+// interface, where two one-sided evaluations per node took 50). 101^3 FP64, all
+// three dimensions: 318 -> 153 us.
+__device__ __forceinline__ float over_dx(float raw, float dx, float) { return raw / dx; }
+// raw / dx by the reciprocal and one Newton correction with the exact residual
+// (the correctly rounded quotient but for rare last bits); not finite: as it is.
+__device__ __forceinline__ double over_dx(double raw, double dx, double inv_dx) {
+    const double q = raw * inv_dx;
+    const double c = fma(fma(-q, dx, raw), inv_dx, q);
+    return (__double2hiint(q) & 0x7ff00000) == 0x7ff00000 ? q : c;
+}
+
+constexpr int kUpwindThreads = 128;
+constexpr int kUpwindRun = 8;
+
+template <typename T, int SCHEME>
+__global__ void __launch_bounds__(kUpwindThreads) upwind_kernel(const UpwindParams P) {
+    constexpr int kLines = sizeof(T) == 4 ? 2 : 1;
+    const int d = P.dim, n = P.g.n[d];
+    const long long s = P.g.stride[d], lines = P.g.total / n, group = (lines + kLines - 1) / kLines;
+    const int runs = (n + 1 + kUpwindRun - 1) / kUpwindRun;
+    const bool periodic = (P.g.periodic_mask >> d) & 1u;
+    const int extrap = P.g.extrap;
     const T* __restrict__ u = static_cast<const T*>(P.u);
-    for (int z = blockIdx.z; z < nz; z += gridDim.z) {
-        int idx[4] = {i0, i1, 0, 0};
-        if (D > 2) { idx[2] = z % g.n[2]; }
-        if (D > 3) { idx[3] = z / g.n[2]; }
-        long long flat = 0;
+    T* __restrict__ pm = static_cast<T*>(P.pm);
+    T* __restrict__ pp = static_cast<T*>(P.pp);
+    const T dx = T(P.dx), inv_dx = T(P.inv_dx), inv_6dx = T(P.inv_6dx), floor = T(P.weno_floor);
+    grid_wait();
+    const long long item = (long long)blockIdx.x * kUpwindThreads + threadIdx.x;
+    if (item >= group * runs) return;
+    // neighbouring threads: neighbouring runs of a row along dimension 0, else neighbouring lines
+    const long long line = d == 0 ? item / runs : item % group;
+    const int j0 = kUpwindRun * (int)(d == 0 ? item % runs : item / group);
+    const int j1 = min(j0 + kUpwindRun, n + 1);
+    long long base[kLines];
 #pragma unroll
-        for (int d = 0; d < D; ++d) flat += (long long)idx[d] * g.stride[d];
-        const int d = P.dim;
-        T v[7], pm, pp;
-        gather7<T>(u, flat, idx[d], g.n[d], g.stride[d], (g.periodic_mask >> d) & 1u, g.extrap, v);
-        upwind_pair<T, SCHEME>(v, g.dx[d], P.inv_6dx, T(P.weno_floor), pm, pp);
-        static_cast<T*>(P.pm)[flat] = pm;
-        static_cast<T*>(P.pp)[flat] = pp;
+    for (int l = 0; l < kLines; ++l) {
+        const long long k = min(line + l * group, lines - 1);  // a last odd line is done twice
+        base[l] = k / s * (s * n) + k % s;
+    }
+    auto at = [&](long long b, int j) -> T {  // node j of a line, ghosts included
+        if (j >= 0 && j < n) return ld(u + b + j * s);
+        if (periodic) {
+            int w = j % n;
+            if (w < 0) w += n;
+            return ld(u + b + w * s);
+        }
+        const T e = ld(u + b + (j < 0 ? 0 : n - 1) * s), i = ld(u + b + (j < 0 ? 1 : n - 2) * s);
+        const T slope = (extrap == HJ_EXTRAP_LINEAR) ? (e - i) : fabs(e - i) * sgn(e);
+        return add_rn(e, mul_rn(T(j < 0 ? -j : j - (n - 1)), slope));
+    };
+    auto store = [&](int j, const T* left, const T* right) {  // interface j: right = p+ of node j-1, left = p- of node j
+#pragma unroll
+        for (int l = 0; l < kLines; ++l) {
+            T a = left[l], b = right[l];
+            if constexpr (SCHEME == HJ_WENO5) {
+                a *= inv_6dx;
+                b *= inv_6dx;
+            } else {
+                a = over_dx(a, dx, inv_dx);
+                b = over_dx(b, dx, inv_dx);
+            }
+            if (j < n) pm[base[l] + j * s] = a;
+            if (j > 0) pp[base[l] + (j - 1) * s] = b;
+        }
+    };
+    T v[kLines][6];  // nodes j-3 .. j+2
+#pragma unroll
+    for (int l = 0; l < kLines; ++l)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[l][k] = at(base[l], j0 - 3 + k);
+    [[maybe_unused]] Weno5Line walk;
+    if constexpr (std::is_same<T, double>::value && SCHEME == HJ_WENO5)
+        walk.start(v[0][0], v[0][1], v[0][2], v[0][3], v[0][4], v[0][5]);
+#pragma unroll 1
+    for (int j = j0;; ++j) {
+        T left[kLines], right[kLines], next[kLines];
+        const bool more = j + 1 < j1;
+        if (more) {
+#pragma unroll
+            for (int l = 0; l < kLines; ++l) next[l] = at(base[l], j + 3);
+        }
+        if constexpr (std::is_same<T, double>::value && SCHEME == HJ_WENO5) walk.eval(floor, right[0], left[0]);
+        else iface_item<SCHEME>(v, floor, right, left);
+        store(j, left, right);
+        if (!more) break;
+        if constexpr (std::is_same<T, double>::value && SCHEME == HJ_WENO5) {
+            walk.slide(v[0][5], next[0]);
+            v[0][5] = next[0];
+        } else {
+#pragma unroll
+            for (int l = 0; l < kLines; ++l) {
+#pragma unroll
+                for (int k = 0; k < 5; ++k) v[l][k] = v[l][k + 1];
+                v[l][5] = next[l];
+            }
+        }
     }
 }
 
@@ -118,16 +198,10 @@ cudaError_t launch_stage_t(const StageParams& p, int scheme, cudaStream_t s) {
 
 template <typename T, int SCHEME>
 cudaError_t launch_upwind_scheme(const UpwindParams& p, cudaStream_t s) {
-    dim3 grid, block;
-    launch_shape(p.g, grid, block);
-    switch (p.g.ndim) {
-    case 1: upwind_kernel<T, 1, SCHEME><<<grid, block, 0, s>>>(p); break;
-    case 2: upwind_kernel<T, 2, SCHEME><<<grid, block, 0, s>>>(p); break;
-    case 3: upwind_kernel<T, 3, SCHEME><<<grid, block, 0, s>>>(p); break;
-    case 4: upwind_kernel<T, 4, SCHEME><<<grid, block, 0, s>>>(p); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    const long long n = p.g.n[p.dim], lines = p.g.total / n, group = sizeof(T) == 4 ? (lines + 1) / 2 : lines;
+    const long long items = group * ((n + 1 + kUpwindRun - 1) / kUpwindRun);
+    return launch_dependent(upwind_kernel<T, SCHEME>, dim3((unsigned)((items + kUpwindThreads - 1) / kUpwindThreads)),
+                            dim3(kUpwindThreads), 0, s, p);
 }
 
 template <typename T>

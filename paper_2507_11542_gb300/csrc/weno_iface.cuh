@@ -308,4 +308,26 @@ __device__ __forceinline__ void iface_line(const double v[7], double floor12, D2
     }
 }
 
+// One interface (FP64) or two (FP32, one per lane) from the values at six nodes.
+template <int SCHEME>
+__device__ __forceinline__ void iface_item(const double (&v)[1][6], double floor12, double* pp, double* pm) {
+    const double* w = v[0];
+    if constexpr (SCHEME == HJ_WENO5)
+        weno_iface(w[1] - w[0], w[2] - w[1], w[3] - w[2], w[4] - w[3], w[5] - w[4], floor12, *pp, *pm);
+    else if constexpr (SCHEME == HJ_ENO1) *pp = *pm = __dsub_rn(w[3], w[2]);
+    else if constexpr (SCHEME == HJ_ENO2) eno2_iface(w[1], w[2], w[3], w[4], *pp, *pm);
+    else eno3_iface(w[0], w[1], w[2], w[3], w[4], w[5], *pp, *pm);
+}
+template <int SCHEME>
+__device__ __forceinline__ void iface_item(const float (&v)[2][6], float floor, float* pp, float* pm) {
+    F2 w[6], p, m;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) w[k] = lanes(v[0][k], v[1][k]);
+    iface_lanes<SCHEME>(w, floor, p, m);
+    pp[0] = lane_a(p);
+    pp[1] = lane_b(p);
+    pm[0] = lane_a(m);
+    pm[1] = lane_b(m);
+}
+
 }  // namespace hj
