@@ -16,7 +16,7 @@ template <> __device__ __forceinline__ float batch_dt<float>(const BatchInst& I)
 
 // KIND: kKindFirst for stage 1, kKindCombine for stages 2 and 3.
 template <typename T, int D, int DYN, int SCHEME, int KIND>
-__global__ void __launch_bounds__(RowsBounds<T, D>::kThreads, 1)
+__global__ void __launch_bounds__(sizeof(T) == 4 ? kRowsThreadsF32 : kRowsThreadsF64, 1)
     batch_kernel(const BatchTile* tiles, const BatchInst* insts, const int stage) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_wait();  // the descriptors change from step to step

@@ -385,7 +385,7 @@ void tile_shape(const Slot& S, int threads, int tz_target, int* sx, int* ty, int
     do {
         *sx = rows_segment(S.G.n[0], *ty, nn);
         nn -= 32;
-    } while (rows_node_threads(*sx, *ty) + rows_edge_threads(*sx) > threads);
+    } while (rows_node_threads(*sx, *ty) + rows_edge_threads(*sx, S.dtype == HJ_F64) > threads);
     const int D = S.G.ndim;
     *tz = D >= 3 ? std::max(1, std::min(tz_target, S.G.n[D - 1])) : 1;
 }
@@ -434,7 +434,7 @@ hj_status Engine::shape_group(Group& g, const std::vector<int>& members, const s
         if (threads <= max_block_threads(g.dtype)) {
             if (g.ndim < 3) cands.push_back({threads, 1});
             else
-                for (int tzt : {4, 8, 16, 32}) cands.push_back({threads, tzt});
+                for (int tzt : {4, 6, 8, 12, 16, 24, 32}) cands.push_back({threads, tzt});
         }
     std::pair<int, int> best = cands[0];
     if (cands.size() > 1) {

@@ -348,7 +348,7 @@ std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtyp
             for (int k = 0; k < (D >= 3 ? (int)(sizeof tzs / sizeof tzs[0]) + 1 : 1); ++k) {
                 const int tz = D < 3 ? 1 : k < (int)(sizeof tzs / sizeof tzs[0]) ? tzs[k] : ns;
                 if (D >= 3 && tz >= ns && k < (int)(sizeof tzs / sizeof tzs[0])) continue;
-                const RowsCfg c = make_rows_cfg(G, sx, ty, tz, rows_node_threads(sx, ty) + rows_edge_threads(sx));
+                const RowsCfg c = make_rows_cfg(G, sx, ty, tz, rows_node_threads(sx, ty) + rows_edge_threads(sx, dtype == HJ_F64));
                 if (c.nchunks > 65535 || c.nt > rows_max_threads(f64)) continue;
                 const int bps = rows_bps(P, c, dtype);
                 if (bps <= 0) continue;
@@ -408,7 +408,7 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
         if (fits) {
             const int ty = std::min(tile[0], kRowsMaxTy);
             const int sx = rows_segment(G.n[0], ty, rows_max_node_threads(dtype == HJ_F64));
-            *out = make_rows_cfg(G, sx, ty, tz, rows_node_threads(sx, ty) + rows_edge_threads(sx));
+            *out = make_rows_cfg(G, sx, ty, tz, rows_node_threads(sx, ty) + rows_edge_threads(sx, dtype == HJ_F64));
             if (out->nchunks <= 65535 && rows_bps(P, *out, dtype) > 0) {
                 ctx->rows_cache[pkey] = *out;
                 return HJ_OK;

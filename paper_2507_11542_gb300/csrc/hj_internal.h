@@ -170,9 +170,16 @@ inline int rows_segment(int n0, int ty, int node_threads) {
     const int nseg = (n0 + most - 1) / most;
     return (n0 + nseg - 1) / nseg;
 }
-// Edge threads beside a tile's node threads: one per column and row pair (their
-// last interfaces, and the halo of their line).
-inline int rows_edge_threads(int sx) { return (sx + 4 + 31) / 32 * 32; }
+// Edge threads beside a tile's node threads (the tile's last interfaces, one per
+// two columns and per row pair, and the halos). A block waits for its edge warps
+// in every plane: with one column of halo a thread the FP32 stage of 101^3 takes
+// 15.6 us, with two (and half the threads) 21; in FP64, whose planes take longer,
+// 240 and 231 us.
+__host__ __device__ constexpr int rows_edge_cols(bool f64) { return f64 ? 2 : 1; }
+inline int rows_edge_threads(int sx, bool f64) {
+    const int need = f64 ? (sx + 1) / 2 + 4 : sx + 4;
+    return (need + 31) / 32 * 32;
+}
 inline RowsCfg make_rows_cfg(const GridDev& G, int sx, int ty, int tz, int nt) {
     RowsCfg c;
     c.sx = sx;

@@ -37,7 +37,7 @@ namespace hj {
 // FP32 stage of 101^3 / 161x113x79 at 640, 768, 896, 1024 threads (96, 80, 72, 64
 // registers): 16.7, 16.1, 15.7, 16.2 / 22.6, 20.5, 20.0, 20.7 us; of 81^4 at 768 and
 // 896: 0.69 and 0.71 ms.
-template <typename T, int D> struct RowsBounds { static constexpr int kThreads = D == 3 ? 896 : 768; };
+template <typename T, int D> struct RowsBounds { static constexpr int kThreads = D == 2 ? 768 : 896; };
 template <int D> struct RowsBounds<double, D> { static constexpr int kThreads = kRowsThreadsF64; };
 
 // The slope that ghost values continue outward, and the m-th ghost value.
@@ -165,26 +165,21 @@ __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __rest
     const int plane0 = (D == 4) ? C.i2 * (int)g.stride[2] : 0;
     const T fl0 = SP<T>::floor(P, 0), fl1 = SP<T>::floor(P, 1);
 
-    // A thread's share of a plane's halo (en >= sx + 4): the rows -3, -2, -1, rv,
-    // rv+1, rv+2 of column et, and for the last eight threads the columns -3,
-    // -2, -1, sx, sx+1, sx+2 of a row. Sources do not change from plane to plane:
-    // a flat index of plane 0, or the distance of a ghost cell from the grid
-    // (extrapolated edges). A ghost cell needs the two outermost values at its
-    // end of the line, which are loaded one plane before they are used.
+    // A thread's share of a plane's halo: the rows -3, -2, -1, rv, rv+1, rv+2 of
+    // kCols columns (et, et + en, ...), and for the last eight threads the columns
+    // -3, -2, -1, sx, sx+1, sx+2 of a row. Sources do not change from plane to
+    // plane. Ghost cells (extrapolated edges) need the two outermost values at
+    // their end of the line, which are loaded one plane before they are made.
+    constexpr int kCols = rows_edge_cols(sizeof(T) == 8);
     struct Line {
         int src[6];        // flat index, or -1: a ghost cell
-        T m[6];            // ghost cell: its distance from the grid
-        int lo0, lo1, hi0, hi1;
         bool lo, hi;       // the line has ghost cells below, above
+        T m_lo, m_hi;      // distance from the grid of the first and the last of them
         T a0, a1, b0, b1;  // its outermost values in the next plane
     };
     auto make_line = [&](Line& l, int first, int last, int n, bool periodic, int base, int step) {
         l.lo = l.hi = false;
         l.a0 = l.a1 = l.b0 = l.b1 = T(0);
-        l.lo0 = base;
-        l.lo1 = base + step;
-        l.hi0 = base + (n - 1) * step;
-        l.hi1 = base + (n - 2) * step;
 #pragma unroll
         for (int h = 0; h < 6; ++h) {
             int i = h < 3 ? first + h - 3 : last + h - 3;  // -3 .. n + 2
@@ -192,71 +187,109 @@ __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __rest
             if (periodic) i += below ? n : above ? -n : 0;
             else if (below) l.lo = true;
             else if (above) l.hi = true;
-            const bool ghost = !periodic && (below || above);
-            l.src[h] = ghost ? -1 : base + i * step;
-            l.m[h] = T(below ? -i : i - (n - 1));
+            l.src[h] = !periodic && (below || above) ? -1 : base + i * step;
         }
+        l.m_lo = T(3 - first);
+        l.m_hi = T(last + 3 - n);
     };
-    auto fetch = [&](Line& l, int p) {
-        const T* __restrict__ plane = u + p * sS;
-        if (l.lo) { l.a0 = ld(plane + l.lo0); l.a1 = ld(plane + l.lo1); }
-        if (l.hi) { l.b0 = ld(plane + l.hi0); l.b1 = ld(plane + l.hi1); }
+    auto fetch = [&](Line& l, int p, int n, int base, int step) {
+        const T* __restrict__ line = u + p * sS + base;
+        if (l.lo) { l.a0 = ld(line); l.a1 = ld(line + step); }
+        if (l.hi) { l.b0 = ld(line + (n - 1) * step); l.b1 = ld(line + (n - 2) * step); }
     };
-    auto put = [&](const Line& l, int p, T* low, T* high, int step) {
+    auto copy = [&](const Line& l, int p, T* low, T* high, int step) {
         const T* __restrict__ plane = u + p * sS;
+#pragma unroll
+        for (int h = 0; h < 6; ++h)
+            if (l.src[h] >= 0) cp_async_elem(h < 3 ? low + h * step : high + (h - 3) * step, plane + l.src[h]);
+    };
+    auto ghosts = [&](const Line& l, T* low, T* high, int step) {
+        if (!l.lo && !l.hi) return;
         const T sa = outward_slope(l.a0, l.a1, extrap), sb = outward_slope(l.b0, l.b1, extrap);
 #pragma unroll
-        for (int h = 0; h < 6; ++h) {
-            T* dst = h < 3 ? low + h * step : high + (h - 3) * step;
-            if (l.src[h] >= 0) cp_async_elem(dst, plane + l.src[h]);
-            else *dst = add_rn(h < 3 ? l.a0 : l.b0, mul_rn(l.m[h], h < 3 ? sa : sb));
-        }
+        for (int h = 0; h < 6; ++h)
+            if (l.src[h] < 0)
+                *(h < 3 ? low + h * step : high + (h - 3) * step) =
+                    h < 3 ? add_rn(l.a0, mul_rn(add_rn(l.m_lo, T(-h)), sa)) : add_rn(l.b0, mul_rn(add_rn(l.m_hi, T(h - 5)), sb));
     };
-    const bool col_job = et < C.sx;
     const int r = et - (en - kRowsMaxTy);
     const bool row_job = r >= 0 && r < C.rv;
-    Line col, row;
-    if (col_job) make_line(col, C.y0, C.y0 + C.rv, ny, per1, plane0 + C.x0 + et, nx);
-    if (row_job) make_line(row, C.x0, C.x0 + C.sx, nx, per0, plane0 + (C.y0 + r) * nx, 1);
+    const int col_base = plane0 + C.x0 + et, row_base = plane0 + (C.y0 + r) * nx;
+    Line col[kCols], row;
+#pragma unroll
+    for (int k = 0; k < kCols; ++k)
+        if (et + k * en < C.sx) make_line(col[k], C.y0, C.y0 + C.rv, ny, per1, col_base + k * en, nx);
+    if (row_job) make_line(row, C.x0, C.x0 + C.sx, nx, per0, row_base, 1);
+    T* const col_lo = smem + (et + 3) * kP + 1;
+    T* const col_hi = smem + (et + 3) * kP + 4 + C.rv;
+    T* const row_lo = smem + 4 + r;
+    T* const row_hi = smem + (C.sx + 3) * kP + 4 + r;
     auto fetch_all = [&](int p) {
-        if (col_job) fetch(col, p);
-        if (row_job) fetch(row, p);
+#pragma unroll
+        for (int k = 0; k < kCols; ++k)
+            if (et + k * en < C.sx) fetch(col[k], p, ny, col_base + k * en, nx);
+        if (row_job) fetch(row, p, nx, row_base, 1);
     };
-    auto stage = [&](int p, T* b) {
-        if (col_job) put(col, p, b + (et + 3) * kP + 1, b + (et + 3) * kP + 4 + C.rv, 1);
-        if (row_job) put(row, p, b + 4 + r, b + (C.sx + 3) * kP + 4 + r, kP);
-        if (p + 1 < C.zend) fetch_all(p + 1);
+    auto copy_all = [&](int p, int o) {
+#pragma unroll
+        for (int k = 0; k < kCols; ++k)
+            if (et + k * en < C.sx) copy(col[k], p, col_lo + o + k * en * kP, col_hi + o + k * en * kP, 1);
+        if (row_job) copy(row, p, row_lo + o, row_hi + o, kP);
+    };
+    auto ghost_all = [&](int o) {
+#pragma unroll
+        for (int k = 0; k < kCols; ++k)
+            if (et + k * en < C.sx) ghosts(col[k], col_lo + o + k * en * kP, col_hi + o + k * en * kP, 1);
+        if (row_job) ghosts(row, row_lo + o, row_hi + o, kP);
     };
 
+    // first two planes: all copies are under way before the first ghost cell waits for its sources
+    const bool second = C.zbeg + 1 < C.zend;
+    copy_all(C.zbeg, 0);
+    if (second) copy_all(C.zbeg + 1, buf);
     fetch_all(C.zbeg);
-    stage(C.zbeg, smem);
-    if (C.zbeg + 1 < C.zend) stage(C.zbeg + 1, smem + buf);
+    ghost_all(0);
+    if (second) {
+        fetch_all(C.zbeg + 1);
+        ghost_all(buf);
+        if (C.zbeg + 2 < C.zend) fetch_all(C.zbeg + 2);
+    }
     cp_async_wait_all();
     block_barrier(C.nt);
 
-    // left-over interfaces: the gap above the last row where no node thread has
-    // it (an even number of rows), then the last one of each row pair
-    const int n_gap = (C.rv & 1) ? 0 : C.sx;
+    // left-over interfaces, two an item: the gap above the last row of two
+    // columns where no node thread has it (an even number of rows), then the last
+    // interface of both rows of a pair
+    const int n_gap = (C.rv & 1) ? 0 : (C.sx + 1) >> 1;
     const int n_item = n_gap + ((C.rv + 1) >> 1);
 #pragma unroll 1
     for (int z = C.zbeg; z < C.zend; ++z) {
-        T* const bz = smem + ((z - C.zbeg) & 1) * buf;
-#pragma unroll 1
-        for (int i = et; i < n_item; i += en) {
-            const bool gap = i < n_gap;
-            const int pr = i - n_gap;
-            const T* w0 = gap ? bz + (i + 3) * kP + 1 + C.rv : bz + C.sx * kP + 4 + 2 * pr;
-            const int step = gap ? 1 : kP, second = gap ? 0 : 1;
+        const int o = ((z - C.zbeg) & 1) * buf;
+        T* const bz = smem + o;
+        if (et < n_item) {  // en >= (sx + 1) / 2 + 4
+            const bool gap = et < n_gap;
+            const int pr = et - n_gap;
+            const T* w0 = gap ? bz + (2 * et + 3) * kP + 1 + C.rv : bz + C.sx * kP + 4 + 2 * pr;
+            const int step = gap ? 1 : kP, second_lane = gap ? kP : 1;  // (an odd last column: a halo column)
             Lanes<T> w[6], pp, pm;
 #pragma unroll
-            for (int k = 0; k < 6; ++k) w[k] = lanes(w0[k * step], w0[k * step + second]);
+            for (int k = 0; k < 6; ++k) w[k] = lanes(w0[k * step], w0[k * step + second_lane]);
             iface_lanes<SCHEME>(w, gap ? fl1 : fl0, pp, pm);
-            if (gap) bz[(i + 3) * kP + kColY + (C.rv >> 1)] = lane_a(pp);
-            else put_lanes(bz + (C.sx + 3) * kP + kColX + 2 * pr, pp);
+            if (gap) {
+                T* const g0 = bz + (2 * et + 3) * kP + kColY + (C.rv >> 1);
+                g0[0] = lane_a(pp);
+                g0[kP] = lane_b(pp);
+            } else {
+                put_lanes(bz + (C.sx + 3) * kP + kColX + 2 * pr, pp);
+            }
         }
         cp_async_wait_all();  // this thread's copies into plane z+1
         block_barrier(C.nt);
-        if (z + 2 < C.zend) stage(z + 2, bz);
+        if (z + 2 < C.zend) {
+            copy_all(z + 2, o);
+            ghost_all(o);
+            if (z + 3 < C.zend) fetch_all(z + 3);
+        }
     }
 }
 
@@ -409,6 +442,18 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
             }
         }
 
+        // the dimension-2 lines of plane z, loaded before phase A covers their latency
+        T v0[D == 4 ? 7 : 1], v1[D == 4 ? 7 : 1];
+        if constexpr (D == 4) {
+            const bool per2 = (g.periodic_mask >> 2) & 1u;
+            gather7<T>(u, (long long)f0, C.i2, g.n[2], g.stride[2], per2, extrap, v0);
+            gather7<T>(u, (long long)f1, C.i2, g.n[2], g.stride[2], per2, extrap, v1);
+            if constexpr (KIND == kKindCombine) {
+                va = ld(vn + f0);
+                vb = ld(vn + f1);
+            }
+        }
+
         // phase A: interfaces of plane z along dimensions 0 and 1
         L pmx, pmy, pp;
         const T* own = bz + s_own;
@@ -450,10 +495,6 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
         }
         if constexpr (D == 4) {
             // dimension 2: both interfaces of each node from a 7-point line
-            T v0[7], v1[7];
-            const bool per2 = (g.periodic_mask >> 2) & 1u;
-            gather7<T>(u, (long long)f0, C.i2, g.n[2], g.stride[2], per2, extrap, v0);
-            gather7<T>(u, (long long)f1, C.i2, g.n[2], g.stride[2], per2, extrap, v1);
             L l[7], pm2, pp2, unused0, unused1;
 #pragma unroll
             for (int k = 0; k < 7; ++k) l[k] = lanes(v0[k], v1[k]);
@@ -465,10 +506,6 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
             if constexpr (uses_coord<D, DYN>(3)) xa[3] = xb[3] = coord(SP<T>::lo(P, 3), z, SP<T>::dx(P, 3));
         }
         if constexpr (D == 3 && uses_coord<D, DYN>(2)) xa[2] = xb[2] = coord(SP<T>::lo(P, 2), z, SP<T>::dx(P, 2));
-        if constexpr (KIND == kKindCombine && !kVnAhead) {
-            va = ld(vn + f0);
-            vb = ld(vn + f1);
-        }
         T S[D], Q[D];
 #pragma unroll
         for (int d = 0; d < D; ++d) { S[d] = lane_a(sm[d]); Q[d] = lane_a(df[d]); }

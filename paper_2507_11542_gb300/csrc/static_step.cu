@@ -131,7 +131,7 @@ bool pick_rows(const StageParams& P, int dtype, int sm_count, RowsCfg* c) {
     const int ty = std::min(D == 2 ? 4 : kRowsMaxTy, G.n[1]);
     const int sx = rows_segment(G.n[0], ty, dtype == HJ_F64 ? 128 : 256);
     const int ns = D >= 3 ? G.n[D - 1] : 1;
-    *c = make_rows_cfg(G, sx, ty, ns, rows_node_threads(sx, ty) + rows_edge_threads(sx));
+    *c = make_rows_cfg(G, sx, ty, ns, rows_node_threads(sx, ty) + rows_edge_threads(sx, dtype == HJ_F64));
     if (D >= 3) {
         const long long per_plane = (long long)c->tiles * (D == 4 ? G.n[2] : 1);
         const long long chunks = (2LL * sm_count + per_plane - 1) / per_plane;
