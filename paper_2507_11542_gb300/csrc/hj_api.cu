@@ -380,8 +380,7 @@ std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtyp
 
 // The launch shape for this grid: measured once per (shape, dtype, dynamics,
 // scheme, dissipation) over the model's best candidates (groups of
-// first-stage launches writing to a scratch buffer, best of two groups), then
-// cached in the context. A tile override {ty, tz, occ, flags} (ty >= 1)
+// first-stage launches writing to a scratch buffer), then cached in the context. A tile override {ty, tz, occ, flags} (ty >= 1)
 // pins the rows and planes instead; it is validated once and cached like a
 // tuned shape.
 hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_t* tile, RowsCfg* out) {
@@ -444,29 +443,41 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
         // clock advances in steps of about two microseconds
         const double per_us = dtype == HJ_F64 ? 4e3 : 4e4;  // nodes a microsecond, roughly
         const int group = (int)std::min(8.0, std::max(1.0, std::ceil(100.0 * per_us / (double)G.total)));
-        float best_ms = 1e30f;
-        for (const RowsCfg& c : cands) {
-            cudaError_t e = rows_launch(ctx, T, c, dtype);  // warm-up
-            float ms_min = 1e30f;
-            for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
+        const auto timed = [&](const RowsCfg& c, int reps, float* ms_min) -> cudaError_t {
+            cudaError_t e = cudaSuccess;
+            for (int rep = 0; rep < reps && e == cudaSuccess; ++rep) {
                 cudaEventRecord(e0, ctx->stream);
                 for (int k = 0; k < group && e == cudaSuccess; ++k) e = rows_launch(ctx, T, c, dtype);
                 cudaEventRecord(e1, ctx->stream);
                 if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-                float ms = 0.f;
-                if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
-                ms_min = std::min(ms_min, ms);
+                float ms = 1e30f;
+                if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+                *ms_min = std::min(*ms_min, ms);
             }
-            if (e != cudaSuccess) {
-                cudaEventDestroy(e0);
-                cudaEventDestroy(e1);
-                return cuda_fail(ctx, e, "tuning launch");
-            }
-            if (ms_min < best_ms) {
-                best_ms = ms_min;
-                best = c;
-            }
+            return e;
+        };
+        // about a millisecond of launches first (an idle GPU's clocks rise meanwhile), every candidate twice,
+        // then the five best again: a pick by one disturbed group cost up to a third of a step
+        cudaError_t e = cudaSuccess;
+        const int warm = (int)std::min(64.0, std::max(1.0, 1000.0 * per_us / (double)G.total));
+        for (int k = 0; k < warm && e == cudaSuccess; ++k) e = rows_launch(ctx, T, cands[0], dtype);
+        std::vector<std::pair<float, size_t>> took;
+        for (size_t i = 0; i < cands.size() && e == cudaSuccess; ++i) {
+            e = rows_launch(ctx, T, cands[i], dtype);  // loads the kernel, fills the caches
+            float ms = 1e30f;
+            if (e == cudaSuccess) e = timed(cands[i], 2, &ms);
+            took.push_back({ms, i});
         }
+        std::sort(took.begin(), took.end());
+        if (took.size() > 5) took.resize(5);
+        for (auto& t : took)
+            if (e == cudaSuccess) e = timed(cands[t.second], 3, &t.first);
+        if (e != cudaSuccess) {
+            cudaEventDestroy(e0);
+            cudaEventDestroy(e1);
+            return cuda_fail(ctx, e, "tuning launch");
+        }
+        best = cands[std::min_element(took.begin(), took.end())->second];
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
     }

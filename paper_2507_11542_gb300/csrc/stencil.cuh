@@ -423,85 +423,95 @@ __device__ __forceinline__ T lf_combine(const StageParams& P, const T* xc, T c, 
 // The Lax-Friedrichs term of a node from the raw (undivided) one-sided
 // derivatives: sums S_d = p-_d + p+_d and differences Q_d = p+_d - p-_d, with
 // h_d = 1/(2 dx_d), so that the mean is h_d S_d and the half difference h_d Q_d.
-// The same formulas as lf_combine, every operation rounded as written (none is
-// left to contraction, so that every kernel that holds this code rounds alike).
-// Scalar in FP32 too: most operations take a value that is the same for the
-// whole block, which a packed one would want in a register pair.
+// lf_combine's formulas with h folded into what multiplies S and Q: most of it
+// does not change along a thread's column, so that a node pays for fewer
+// operations (air3D: 22 instead of 29, each 16-20 cycles an SM in FP64). Every
+// operation is rounded as written (none is left to contraction, so that every
+// kernel that holds this code rounds alike). Scalar in FP32 too: most operations
+// take a value that is the same for the whole block, which a packed one would
+// want in a register pair.
 template <typename T, int D, int DYN>
 __device__ __forceinline__ T lf_node(const StageParams& P, const T* par, const T* x, T c, T s, const T* S, const T* Q,
                                      const T* h, bool alpha_global) {
     const auto q = [par](int k) { return par[k]; };  // the dynamics' parameters, read once per thread
     constexpr int B = dyn_base(DYN);
-    T pb[D], dd[D], a[D];
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-        pb[d] = mul_rn(S[d], h[d]);
-        dd[d] = mul_rn(Q[d], h[d]);
-        a[d] = T(0);
-    }
+    T a[D];  // h_d alpha_d
     T y;
     if constexpr (B == HJ_DYN_DOUBLE_INTEGRATOR && D == 2) {
-        y = fma_rn(-q(0), absv(pb[1]), mul_rn(pb[0], x[1]));
-        a[0] = absv(x[1]);
-        a[1] = q(0);
+        const T f0 = mul_rn(x[1], h[0]), g1 = mul_rn(q(0), h[1]);
+        y = fma_rn(-g1, absv(S[1]), mul_rn(S[0], f0));
+        a[0] = absv(f0);
+        a[1] = g1;
     } else if constexpr (B == HJ_DYN_AIR3D && D == 3) {
         const T amax = q(2), bmax = q(3);
-        const T f0 = fma_rn(q(1), c, -q(0)), f1 = mul_rn(q(1), s);
-        const T k = fma_rn(x[0], pb[1], fma_rn(-x[1], pb[0], pb[2]));  // its sign does not matter
-        y = fma_rn(pb[1], f1, mul_rn(pb[0], f0));
-        y = fma_rn(-bmax, absv(pb[2]), fma_rn(amax, absv(k), y));
-        a[0] = fma_rn(amax, absv(x[1]), absv(f0));
-        a[1] = fma_rn(amax, absv(x[0]), absv(f1));
-        a[2] = add_rn(amax, bmax);
+        const T f0 = fma_rn(mul_rn(q(1), h[0]), c, -mul_rn(q(0), h[0])), f1 = mul_rn(mul_rn(q(1), h[1]), s);
+        const T x0 = mul_rn(x[0], h[1]), x1 = mul_rn(x[1], h[0]), p2 = mul_rn(S[2], h[2]);
+        const T k = fma_rn(x0, S[1], fma_rn(-x1, S[0], p2));  // its sign does not matter
+        y = fma_rn(S[1], f1, mul_rn(S[0], f0));
+        y = fma_rn(-bmax, absv(p2), fma_rn(amax, absv(k), y));
+        a[0] = add_rn(mul_rn(amax, absv(x1)), absv(f0));
+        a[1] = add_rn(mul_rn(amax, absv(x0)), absv(f1));
+        a[2] = mul_rn(add_rn(amax, bmax), h[2]);
     } else if constexpr (B == HJ_DYN_ROCKETS && D == 3) {
-        const T ac = q(0), g = q(1), ue = q(2), up = q(3);
-        const T f0 = mul_rn(ac, c), f1 = add_rn(fma_rn(ac, s, ac), -g);
-        const T ke = fma_rn(-x[0], pb[0], pb[2]), kp = fma_rn(x[0], pb[1], pb[2]);
-        y = fma_rn(pb[1], f1, mul_rn(pb[0], f0));
+        const T ac = q(0), ue = q(2), up = q(3), ac1 = mul_rn(ac, h[1]);
+        const T f0 = mul_rn(mul_rn(ac, h[0]), c), f1 = fma_rn(ac1, s, mul_rn(add_rn(ac, -q(1)), h[1]));
+        const T xe = mul_rn(x[0], h[0]), xp = mul_rn(x[0], h[1]), p2 = mul_rn(S[2], h[2]);
+        const T ke = fma_rn(-xe, S[0], p2), kp = fma_rn(xp, S[1], p2);
+        y = fma_rn(S[1], f1, mul_rn(S[0], f0));
         y = fma_rn(-up, absv(kp), fma_rn(ue, absv(ke), y));
-        a[0] = fma_rn(ue, absv(x[0]), absv(f0));
-        a[1] = fma_rn(up, absv(x[0]), absv(f1));
-        a[2] = add_rn(ue, up);
+        a[0] = add_rn(mul_rn(ue, absv(xe)), absv(f0));
+        a[1] = add_rn(mul_rn(up, absv(xp)), absv(f1));
+        a[2] = mul_rn(add_rn(ue, up), h[2]);
     } else if constexpr (B == HJ_DYN_DUBINS4D && D == 4) {
-        const T wmax = q(0), accmax = q(1);
-        const T f0 = mul_rn(x[3], c), f1 = mul_rn(x[3], s);
-        y = fma_rn(pb[1], f1, mul_rn(pb[0], f0));
-        y = fma_rn(-accmax, absv(pb[3]), fma_rn(-wmax, absv(pb[2]), y));
+        const T f0 = mul_rn(x[3], mul_rn(c, h[0])), f1 = mul_rn(x[3], mul_rn(s, h[1]));
         a[0] = absv(f0);
         a[1] = absv(f1);
-        a[2] = wmax;
-        a[3] = accmax;
+        a[2] = mul_rn(q(0), h[2]);
+        a[3] = mul_rn(q(1), h[3]);
+        y = fma_rn(S[1], f1, mul_rn(S[0], f0));
+        y = fma_rn(-a[3], absv(S[3]), fma_rn(-a[2], absv(S[2]), y));
     } else if constexpr (B == HJ_DYN_NORM) {
-        T s2 = mul_rn(pb[0], pb[0]);
-        a[0] = q(0);
+        T s2 = T(0);
 #pragma unroll
-        for (int d = 1; d < D; ++d) {
-            s2 = fma_rn(pb[d], pb[d], s2);
-            a[d] = q(0);
+        for (int d = 0; d < D; ++d) {
+            const T p = mul_rn(S[d], h[d]);
+            s2 = d == 0 ? mul_rn(p, p) : fma_rn(p, p, s2);
+            a[d] = mul_rn(q(0), h[d]);
         }
         y = mul_rn(-q(0), sqrt(s2));
     } else if constexpr (B == HJ_DYN_ADVECT) {
-        y = mul_rn(-q(0), pb[0]);
-        a[0] = absv(q(0));
 #pragma unroll
-        for (int d = 1; d < D; ++d) {
-            y = fma_rn(-q(d), pb[d], y);
-            a[d] = absv(q(d));
+        for (int d = 0; d < D; ++d) {
+            const T f = mul_rn(q(d), h[d]);
+            y = d == 0 ? mul_rn(-f, S[d]) : fma_rn(-f, S[d], y);
+            a[d] = absv(f);
         }
     } else {
         static_assert(B == HJ_DYN_ROTATE && D >= 2, "a dynamics of the row kernel");
-        const T f0 = mul_rn(q(0), x[1]), f1 = mul_rn(q(0), x[0]);  // the speeds are -f0, f1
-        y = fma_rn(-f1, pb[1], mul_rn(f0, pb[0]));
+        const T f0 = mul_rn(mul_rn(q(0), x[1]), h[0]), f1 = mul_rn(mul_rn(q(0), x[0]), h[1]);  // the speeds are -f0, f1
+        y = fma_rn(-f1, S[1], mul_rn(f0, S[0]));
         a[0] = absv(f0);
         a[1] = absv(f1);
+#pragma unroll
+        for (int d = 2; d < D; ++d) a[d] = T(0);
     }
-    if constexpr (dyn_is_box(DYN)) box_alpha<T, D, B>(P, x, c, s, pb, dd, a);
+    if constexpr (dyn_is_box(DYN)) {
+        T pb[D], dd[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            pb[d] = mul_rn(S[d], h[d]);
+            dd[d] = mul_rn(Q[d], h[d]);
+        }
+        box_alpha<T, D, B>(P, x, c, s, pb, dd, a);
+#pragma unroll
+        for (int d = 0; d < D; ++d) a[d] = mul_rn(a[d], h[d]);
+    }
     if (alpha_global) {
 #pragma unroll
-        for (int d = 0; d < D; ++d) a[d] = SP<T>::alpha_g(P, d);
+        for (int d = 0; d < D; ++d) a[d] = mul_rn(SP<T>::alpha_g(P, d), h[d]);
     }
 #pragma unroll
-    for (int d = 0; d < D; ++d) y = fma_rn(a[d], dd[d], y);
+    for (int d = 0; d < D; ++d) y = fma_rn(a[d], Q[d], y);
     return y;
 }
 
