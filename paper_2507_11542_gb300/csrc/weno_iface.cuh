@@ -116,9 +116,10 @@ __device__ __forceinline__ double rcp_newton(double x) {
 // 1/(2 dx) (iface_times6). A non-finite difference reaches both results
 // through T1 or T2, since the weights are finite whatever their input.
 //
-// The FP64 pipe bounds this (16-20 cycles a warp instruction and SM): 25 FP64
-// instructions from five first differences, 15 along a line (Weno5Line), where
-// the weights in FP64 took 64 and 50 (1272 and 1009 cycles, now 540 and 340).
+// The FP64 pipe bounds this (16-20 cycles a warp instruction and SM): 22 FP64
+// instructions from five first differences, 12 along a line (Weno5Line), where
+// the weights in FP64 took 64 and 50 (measured cycles per warp and SM in
+// weno_weights64.cuh).
 // The core takes what consecutive interfaces along a line share: tA, tB, tC
 // (the second differences of the windows' first differences), d23, d34 and the
 // third differences T1 = tA - tB, T2 = tB - tC. floor12: 12 times the epsilon
@@ -128,15 +129,15 @@ __device__ __forceinline__ double rcp_newton(double x) {
 __device__ __forceinline__ void weno_core(double e1, double e2, double e3, double e4, double e5, double tA, double tB,
                                           double tC, double d23, double d34, double T1, double T2, double floor12,
                                           double& pp_j, double& pm_j1) {
-    const double uA = fma(2.0, d23, tA);   // e1 - 4e2 + 3e3
-    const double uB = e2 - e4;
-    const double uC = fma(-2.0, d34, tC);  // 3e3 - 4e4 + e5
     const w64::u64 amax = w64::umax(w64::umax(w64::umax(w64::abs_bits(e1), w64::abs_bits(e2)),
                                               w64::umax(w64::abs_bits(e3), w64::abs_bits(e4))), w64::abs_bits(e5));
     const w64::Sum eps = w64::eps_sum(amax, w64::floor_term(floor12));
     double l1, l3, r1, r3;
-    w64::weights(w64::smooth_sum(tA, uA, eps), w64::smooth_sum(tB, uB, eps), w64::smooth_sum(tC, uC, eps), l1, l3, r1,
-                 r3);
+    // u: tA + 2 d23 = e1 - 4e2 + 3e3, d23 + d34 = e4 - e2, tC - 2 d34 = 3e3 - 4e4 + e5
+    const w64::Parts pA = w64::parts(tA), pB = w64::parts(tB), pC = w64::parts(tC), p23 = w64::parts(d23),
+                     p34 = w64::parts(d34);
+    w64::weights(w64::smooth_sum(pA, pA, p23, 1, 0u, eps), w64::smooth_sum(pB, p23, p34, 0, 0u, eps),
+                 w64::smooth_sum(pC, pC, p34, 1, ~0u, eps), l1, l3, r1, r3);
     const double sL = fma(l3, T2, fma(l1, T1, fma(2.0, d34, d23)));
     const double sR = fma(r3, T2, fma(r1, T1, fma(2.0, d23, d34)));
     pm_j1 = fma(6.0, e3, sL);

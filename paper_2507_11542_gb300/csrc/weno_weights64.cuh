@@ -7,8 +7,9 @@
 // numbers and two reciprocals: with 63-bit integer mantissas and integer
 // exponents they need no FP64 instruction, and keep more bits than FP64 does
 // (every product is good to 2^-58 or better, so the weights' error is
-// their final rounding to FP64). Measured on a column sweep that lives in L2:
-// 1009 SM cycles per warp interface with FP64 weights, 340 with these.
+// their final rounding to FP64). Measured on a sweep over columns in L2, SM
+// cycles per warp interface: from six values 1272 with FP64 weights and 460 with
+// these, along a line (Weno5Line) 1009 and 298.
 //
 // A number is a mantissa m < 2^63 and an exponent x; products drop the low
 // partial product (an error below two units of a result of at least 2^58).
@@ -146,15 +147,36 @@ HJ_W64 Sum eps_sum(u64 amax, Sum fl) {
     return {(ka >> imin(x - xa, 63)) + (fl.m >> imin(x - fl.x, 63)), x};
 }
 
-// 12 (S + eps) = 13 t^2 + 3 u^2 + 12 eps, added up as sixteenths (13/16 = 1 -
-// 3/16) so that each term is cut off once: relative error below 2^-54.
-HJ_W64 Sum smooth_sum(double t, double u, Sum eps) {
-    const u64 bt = bits(t), bu = bits(u);
-    const u64 tt = sqrhi(mant(bt)), uu = sqrhi(mant(bu));
-    const int xt = 2 * expo(bt), xu = 2 * expo(bu);
-    const int x = imax(imax(xt, xu), eps.x);
-    const u64 s = ((tt - ((3 * tt) >> 4)) >> imin(x - xt, 63)) + ((3 * uu) >> imin(x - xu + 4, 63)) +
-                  (eps.m >> imin(x - eps.x + 4, 63));  // [2^56, 2^63)
+// A double as a 62-bit mantissa in [2^61, 2^62) and a biased exponent, and its sign.
+struct Parts {
+    u64 m;
+    int x;
+    u32 sign;  // 0 or all ones
+};
+HJ_W64 Parts parts(double d) {
+    const u64 b = bits(d);
+    return {((b << 9) & 0x1fffffffffffffffull) | 0x2000000000000000ull, expo(b), (u32)((int32_t)hi(b) >> 31)};
+}
+
+// 12 (S + eps) = 13 t^2 + 3 u^2 + 12 eps with u = a + 2^k b (flip: a - 2^k b), added
+// up as sixteenths (13/16 = 1 - 3/16) so that each term is cut off once. u is not
+// normalised after a cancellation: a (or t = a) is then as large as 2^k b, so that
+// t^2 or, for the middle window, whose t is the difference of what u adds, the
+// other square carries the sum. Relative error below 2^-54.
+HJ_W64 Sum smooth_sum(Parts t, Parts a, Parts b, int k, u32 flip, Sum eps) {
+    const int xb = b.x + k;
+    const int xu = imax(a.x, xb);
+    const u64 am = a.m >> imin(xu - a.x, 63), bm = b.m >> imin(xu - xb, 63);
+    const u32 sub = a.sign ^ b.sign ^ flip;         // all ones: the magnitudes are subtracted
+    const u64 subw = (u64)sub << 32 | sub;
+    const u64 sum = am + (bm ^ subw) + (sub & 1u);   // below 2^63, or negative
+    const u32 neg = (u32)((int32_t)hi(sum) >> 31);
+    const u64 negw = (u64)neg << 32 | neg;
+    const u64 tt = sqrhi(t.m), uu = sqrhi((sum ^ negw) + (neg & 1u));
+    const int xt2 = 2 * t.x + 2, xu2 = 2 * xu + 2;
+    const int x = imax(imax(xt2, xu2), eps.x);
+    const u64 s = ((tt - ((3 * tt) >> 4)) >> imin(x - xt2, 63)) + ((3 * uu) >> imin(x - xu2 + 4, 63)) +
+                  (eps.m >> imin(x - eps.x + 4, 63));
     const int n = clz(hi(s)) - 1;
     return {s << n, x - n + 4};
 }
