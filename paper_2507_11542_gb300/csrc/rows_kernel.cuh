@@ -373,11 +373,13 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
     // Streamed-dimension queue: q[k] = V at plane z-2+k (k = 0..5); carry = raw p- at z.
     // A warm-up step evaluates the interface below the first plane, so that
     // every interface goes through the same code and results do not depend
-    // on where chunks start. FP64 WENO5 keeps the differences instead
-    // (Weno5Line, bit for bit the same results).
+    // on where chunks start. FP64 WENO5 and ENO2 keep the differences instead
+    // (Weno5Line, Eno2Line; bit for bit the same results).
     constexpr bool kSlide = std::is_same<T, double>::value && SCHEME == HJ_WENO5 && D >= 3;
     L q[6], q6{}, carry{};
-    Weno5Line za, zb;
+    constexpr bool kSlide2 = std::is_same<T, double>::value && SCHEME == HJ_ENO2 && D >= 3;
+    [[maybe_unused]] Weno5Line za, zb;
+    [[maybe_unused]] Eno2Line ea, eb;
     if constexpr (D >= 3) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) q[k] = column(C.zbeg - 3 + k);
@@ -387,6 +389,11 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
             za.eval(flS, unused.a, carry.a);
             zb.start(q[0].b, q[1].b, q[2].b, q[3].b, q[4].b, q[5].b);
             zb.eval(flS, unused.b, carry.b);
+        } else if constexpr (kSlide2) {
+            ea.start(q[1].a, q[2].a, q[3].a, q[4].a);
+            ea.eval(unused.a, carry.a);
+            eb.start(q[1].b, q[2].b, q[3].b, q[4].b);
+            eb.eval(unused.b, carry.b);
         } else {
             iface_lanes<SCHEME>(q, flS, unused, carry);
         }
@@ -486,6 +493,11 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
                 za.eval(flS, pps.a, next.a);
                 zb.slide(q[4].b, q[5].b);
                 zb.eval(flS, pps.b, next.b);
+            } else if constexpr (kSlide2) {
+                ea.slide(q[3].a, q[4].a);
+                ea.eval(pps.a, next.a);
+                eb.slide(q[3].b, q[4].b);
+                eb.eval(pps.b, next.b);
             } else {
                 iface_lanes<SCHEME>(q, flS, pps, next);
             }

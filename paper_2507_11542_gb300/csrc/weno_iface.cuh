@@ -217,6 +217,33 @@ __device__ __forceinline__ void eno2_iface(T v0, T v1, T v2, T v3, T& pp_j, T& p
     pm_j1 = e + T(0.5) * c;
 }
 
+// FP64 ENO2 along a grid line: each interface takes two of its three first and
+// one of its two second differences from the one below it (4 FP64 instructions
+// instead of 7), the results of eno2_iface bit for bit.
+struct Eno2Line {
+    double e, r, dR;  // v2 - v1, v3 - v2, and the second difference between them
+    double dL;
+    // the window of the values v0..v3 at nodes j-1 .. j+2
+    __device__ __forceinline__ void start(double v0, double v1, double v2, double v3) {
+        e = v2 - v1;
+        r = v3 - v2;
+        dL = e - (v1 - v0);
+        dR = r - e;
+    }
+    // slide by one node: v3, v4 are the values at the new window's last two nodes
+    __device__ __forceinline__ void slide(double v3, double v4) {
+        e = r;
+        dL = dR;
+        r = v4 - v3;
+        dR = r - e;
+    }
+    __device__ __forceinline__ void eval(double& pp_j, double& pm_j1) const {
+        const double c = abs_le(dL, dR) ? dL : dR;
+        pp_j = fma(-0.5, c, e);
+        pm_j1 = fma(0.5, c, e);
+    }
+};
+
 // Third-order ENO (Sec. 3.2; Osher & Fedkiw 2003 Sec. 3.3) per interface.
 // p+ of node j and p- of node j+1 both start from k = j, so they take the
 // same second-difference choice (c; k* = j-1 on the left, else j) and the
