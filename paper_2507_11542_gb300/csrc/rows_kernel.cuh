@@ -43,7 +43,9 @@ template <int D> struct RowsBounds<double, D> { static constexpr int kThreads = 
 // The slope that ghost values continue outward, and the m-th ghost value.
 template <typename T>
 __device__ __forceinline__ T outward_slope(T edge, T inner, int extrap) {
-    return (extrap == HJ_EXTRAP_LINEAR) ? (edge - inner) : fabs(edge - inner) * sgn(edge);
+    const T d = edge - inner;
+    if (extrap == HJ_EXTRAP_LINEAR) return d;
+    return edge == T(0) ? fabs(d) * T(0) : copysign(d, edge);
 }
 template <typename T>
 __device__ __forceinline__ T ghost_value(T edge, T inner, int m, int extrap) {
@@ -165,82 +167,93 @@ __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __rest
     const int plane0 = (D == 4) ? C.i2 * (int)g.stride[2] : 0;
     const T fl0 = SP<T>::floor(P, 0), fl1 = SP<T>::floor(P, 1);
 
-    // A thread's share of a plane's halo: the rows -3, -2, -1, rv, rv+1, rv+2 of
-    // kCols columns (et, et + en, ...), and for the last eight threads the columns
-    // -3, -2, -1, sx, sx+1, sx+2 of a row. Sources do not change from plane to
+    // A thread's share of a plane's halo: the rows -3, -2, -1 and rv, rv+1, rv+2 of
+    // kCols columns (et, et + en, ...), and for the last sixteen threads the columns
+    // -3, -2, -1 or sx, sx+1, sx+2 of a row. Sources do not change from plane to
     // plane. Ghost cells (extrapolated edges) need the two outermost values at
-    // their end of the line, which are loaded one plane before they are made.
+    // their end of the line, which are loaded one plane before they are made. In a
+    // launch of one wave the blocks that make them take the longest: this path is
+    // kept short.
     constexpr int kCols = rows_edge_cols(sizeof(T) == 8);
-    struct Line {
-        int src[6];        // flat index, or -1: a ghost cell
-        bool lo, hi;       // the line has ghost cells below, above
-        T m_lo, m_hi;      // distance from the grid of the first and the last of them
-        T a0, a1, b0, b1;  // its outermost values in the next plane
+    struct Side {
+        int src[3];  // flat index, or -1: a ghost cell
+        bool ghost;  // the side has ghost cells
+        T m;         // distance of its first cell from the grid
+        T e, i;      // outermost values in the next plane
     };
-    auto make_line = [&](Line& l, int first, int last, int n, bool periodic, int base, int step) {
-        l.lo = l.hi = false;
-        l.a0 = l.a1 = l.b0 = l.b1 = T(0);
+    auto make_side = [&](Side& q, int first, int n, bool periodic, int base, int step, bool high) {
+        q.ghost = false;
+        q.e = q.i = T(0);
+        q.m = T(high ? first - (n - 1) : -first);
 #pragma unroll
-        for (int h = 0; h < 6; ++h) {
-            int i = h < 3 ? first + h - 3 : last + h - 3;  // -3 .. n + 2
-            const bool below = i < 0, above = i >= n;
-            if (periodic) i += below ? n : above ? -n : 0;
-            else if (below) l.lo = true;
-            else if (above) l.hi = true;
-            l.src[h] = !periodic && (below || above) ? -1 : base + i * step;
+        for (int h = 0; h < 3; ++h) {
+            int i = first + h;  // -3 .. n + 2
+            const bool out = i < 0 || i >= n;
+            if (periodic) i += i < 0 ? n : i >= n ? -n : 0;
+            else if (out) q.ghost = true;
+            q.src[h] = !periodic && out ? -1 : base + i * step;
         }
-        l.m_lo = T(3 - first);
-        l.m_hi = T(last + 3 - n);
     };
-    auto fetch = [&](Line& l, int p, int n, int base, int step) {
-        const T* __restrict__ line = u + p * sS + base;
-        if (l.lo) { l.a0 = ld(line); l.a1 = ld(line + step); }
-        if (l.hi) { l.b0 = ld(line + (n - 1) * step); l.b1 = ld(line + (n - 2) * step); }
+    auto fetch = [&](Side& q, const T* __restrict__ line, int n, int step, bool high) {
+        if (q.ghost) {
+            q.e = ld(line + (high ? (n - 1) * step : 0));
+            q.i = ld(line + (high ? (n - 2) * step : step));
+        }
     };
-    auto copy = [&](const Line& l, int p, T* low, T* high, int step) {
-        const T* __restrict__ plane = u + p * sS;
+    auto copy = [&](const Side& q, const T* __restrict__ plane, T* dst, int step) {
 #pragma unroll
-        for (int h = 0; h < 6; ++h)
-            if (l.src[h] >= 0) cp_async_elem(h < 3 ? low + h * step : high + (h - 3) * step, plane + l.src[h]);
+        for (int h = 0; h < 3; ++h)
+            if (q.src[h] >= 0) cp_async_elem(dst + h * step, plane + q.src[h]);
     };
-    auto ghosts = [&](const Line& l, T* low, T* high, int step) {
-        if (!l.lo && !l.hi) return;
-        const T sa = outward_slope(l.a0, l.a1, extrap), sb = outward_slope(l.b0, l.b1, extrap);
+    auto ghosts = [&](const Side& q, T* dst, int step, T dir) {  // dir: 1 above the grid, -1 below
+        if (!q.ghost) return;
+        const T slope = outward_slope(q.e, q.i, extrap);
 #pragma unroll
-        for (int h = 0; h < 6; ++h)
-            if (l.src[h] < 0)
-                *(h < 3 ? low + h * step : high + (h - 3) * step) =
-                    h < 3 ? add_rn(l.a0, mul_rn(add_rn(l.m_lo, T(-h)), sa)) : add_rn(l.b0, mul_rn(add_rn(l.m_hi, T(h - 5)), sb));
+        for (int h = 0; h < 3; ++h)
+            if (q.src[h] < 0) dst[h * step] = add_rn(q.e, mul_rn(fma_rn(dir, T(h), q.m), slope));
     };
-    const int r = et - (en - kRowsMaxTy);
-    const bool row_job = r >= 0 && r < C.rv;
+    const int rt = et - (en - 2 * kRowsMaxTy), r = rt & (kRowsMaxTy - 1);
+    const bool row_high = rt >= kRowsMaxTy, row_job = rt >= 0 && r < C.rv;
     const int col_base = plane0 + C.x0 + et, row_base = plane0 + (C.y0 + r) * nx;
-    Line col[kCols], row;
+    Side low[kCols], high[kCols], row;
 #pragma unroll
     for (int k = 0; k < kCols; ++k)
-        if (et + k * en < C.sx) make_line(col[k], C.y0, C.y0 + C.rv, ny, per1, col_base + k * en, nx);
-    if (row_job) make_line(row, C.x0, C.x0 + C.sx, nx, per0, row_base, 1);
-    T* const col_lo = smem + (et + 3) * kP + 1;
-    T* const col_hi = smem + (et + 3) * kP + 4 + C.rv;
-    T* const row_lo = smem + 4 + r;
-    T* const row_hi = smem + (C.sx + 3) * kP + 4 + r;
+        if (et + k * en < C.sx) {
+            make_side(low[k], C.y0 - 3, ny, per1, col_base + k * en, nx, false);
+            make_side(high[k], C.y0 + C.rv, ny, per1, col_base + k * en, nx, true);
+        }
+    if (row_job) make_side(row, row_high ? C.x0 + C.sx : C.x0 - 3, nx, per0, row_base, 1, row_high);
+    T* const col_low = smem + (et + 3) * kP + 1;
+    T* const col_high = smem + (et + 3) * kP + 4 + C.rv;
+    T* const row_to = smem + (row_high ? (C.sx + 3) * kP : 0) + 4 + r;
     auto fetch_all = [&](int p) {
+        const T* __restrict__ plane = u + p * sS;
 #pragma unroll
         for (int k = 0; k < kCols; ++k)
-            if (et + k * en < C.sx) fetch(col[k], p, ny, col_base + k * en, nx);
-        if (row_job) fetch(row, p, nx, row_base, 1);
+            if (et + k * en < C.sx) {
+                fetch(low[k], plane + col_base + k * en, ny, nx, false);
+                fetch(high[k], plane + col_base + k * en, ny, nx, true);
+            }
+        if (row_job) fetch(row, plane + row_base, nx, 1, row_high);
     };
     auto copy_all = [&](int p, int o) {
+        const T* __restrict__ plane = u + p * sS;
 #pragma unroll
         for (int k = 0; k < kCols; ++k)
-            if (et + k * en < C.sx) copy(col[k], p, col_lo + o + k * en * kP, col_hi + o + k * en * kP, 1);
-        if (row_job) copy(row, p, row_lo + o, row_hi + o, kP);
+            if (et + k * en < C.sx) {
+                copy(low[k], plane, col_low + o + k * en * kP, 1);
+                copy(high[k], plane, col_high + o + k * en * kP, 1);
+            }
+        if (row_job) copy(row, plane, row_to + o, kP);
     };
     auto ghost_all = [&](int o) {
 #pragma unroll
         for (int k = 0; k < kCols; ++k)
-            if (et + k * en < C.sx) ghosts(col[k], col_lo + o + k * en * kP, col_hi + o + k * en * kP, 1);
-        if (row_job) ghosts(row, row_lo + o, row_hi + o, kP);
+            if (et + k * en < C.sx) {
+                ghosts(low[k], col_low + o + k * en * kP, 1, T(-1));
+                ghosts(high[k], col_high + o + k * en * kP, 1, T(1));
+            }
+        if (row_job) ghosts(row, row_to + o, kP, row_high ? T(1) : T(-1));
     };
 
     // first two planes: all copies are under way before the first ghost cell waits for its sources
