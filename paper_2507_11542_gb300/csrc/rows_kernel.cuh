@@ -153,7 +153,7 @@ constexpr int kColX = 16, kColY = 24;
 // into the means and half differences the Hamiltonian takes. Flat indices are
 // 32-bit (the grid has fewer than 2^31 nodes). Threads of the node warps
 // without a node work on a clamped one and store nothing.
-template <typename T, int D, int SCHEME>
+template <typename T, int D, int SCHEME, bool WAIT>
 __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __restrict__ u, const Tile& C, const int t,
                                            T* const smem, const int buf) {
     constexpr int kP = kRowsPitch;
@@ -236,6 +236,16 @@ __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __rest
             }
         if (row_job) fetch(row, plane + row_base, nx, 1, row_high);
     };
+    auto keep = [&](Side* to) {  // the values fetched last
+#pragma unroll
+        for (int k = 0; k < kCols; ++k) { to[2 * k] = low[k]; to[2 * k + 1] = high[k]; }
+        to[2 * kCols] = row;
+    };
+    auto use = [&](const Side* from) {
+#pragma unroll
+        for (int k = 0; k < kCols; ++k) { low[k] = from[2 * k]; high[k] = from[2 * k + 1]; }
+        row = from[2 * kCols];
+    };
     auto copy_all = [&](int p, int o) {
         const T* __restrict__ plane = u + p * sS;
 #pragma unroll
@@ -256,16 +266,27 @@ __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __rest
         if (row_job) ghosts(row, row_to + o, kP, row_high ? T(1) : T(-1));
     };
 
-    // first two planes: all copies are under way before the first ghost cell waits for its sources
+    // first two planes: all copies and all sources are under way before the first ghost cell waits for its own
+    if constexpr (WAIT) grid_wait();
     const bool second = C.zbeg + 1 < C.zend;
+    Side first[2 * kCols + 1], next[2 * kCols + 1];
     copy_all(C.zbeg, 0);
     if (second) copy_all(C.zbeg + 1, buf);
     fetch_all(C.zbeg);
-    ghost_all(0);
+    keep(first);
     if (second) {
         fetch_all(C.zbeg + 1);
-        ghost_all(buf);
+        keep(next);
         if (C.zbeg + 2 < C.zend) fetch_all(C.zbeg + 2);
+        Side third[2 * kCols + 1];
+        keep(third);
+        use(next);
+        ghost_all(buf);
+        use(first);
+        ghost_all(0);
+        use(third);
+    } else {
+        ghost_all(0);
     }
     cp_async_wait_all();
     block_barrier(C.nt);
@@ -306,7 +327,7 @@ __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __rest
     }
 }
 
-template <typename T, int D, int DYN, int SCHEME, int KIND>
+template <typename T, int D, int DYN, int SCHEME, int KIND, bool WAIT>
 __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<T>& R, const Tile& C, const int t,
                                            T* const smem, const int buf) {
     using L = Lanes<T>;
@@ -371,6 +392,7 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
         xb[1] = coord(SP<T>::lo(P, 1), y1, SP<T>::dx(P, 1));
     }
     if constexpr (D == 4 && uses_coord<D, DYN>(2)) xa[2] = xb[2] = coord(SP<T>::lo(P, 2), C.i2, SP<T>::dx(P, 2));
+    if constexpr (WAIT) grid_wait();
     const T* __restrict__ trig = Trig<T>::get(P);       // cos of the dimension-2 coordinate
     const T* __restrict__ trig_s = uses_angle<D, DYN>() ? trig + g.n[2] : trig;  // sin
     T cos2 = T(0), sin2 = T(0);  // angle of dimension 2 (fixed for the block in 4-D, the next plane's in 3-D)
@@ -553,7 +575,7 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
     }
 }
 
-template <typename T, int D, int DYN, int SCHEME, int KIND>
+template <typename T, int D, int DYN, int SCHEME, int KIND, bool WAIT = false>
 __device__ __forceinline__ void rows_tile(const StageParams& P, const StageRun<T>& R, const int SX, const int TY,
                                           const int NT, const int tz, const int tile, const int i2, const int chunk,
                                           const int t, T* const smem) {
@@ -573,8 +595,8 @@ __device__ __forceinline__ void rows_tile(const StageParams& P, const StageRun<T
     C.nn = rows_node_threads(SX, TY);
     C.nt = NT;
     const int buf = rows_buf_elems(SX);
-    if (t < C.nn) node_warps<T, D, DYN, SCHEME, KIND>(P, R, C, t, smem, buf);
-    else edge_warps<T, D, SCHEME>(P, R.u, C, t, smem, buf);
+    if (t < C.nn) node_warps<T, D, DYN, SCHEME, KIND, WAIT>(P, R, C, t, smem, buf);
+    else edge_warps<T, D, SCHEME, WAIT>(P, R.u, C, t, smem, buf);
 }
 
 template <typename T, int D, int DYN, int SCHEME, int KIND>
@@ -583,8 +605,7 @@ __global__ void __launch_bounds__(RowsBounds<T, D>::kThreads, 1) rows_kernel(con
     const StageRun<T> R = stage_run<T>(P);
     const int i2 = (D == 4) ? (int)blockIdx.y : 0;
     const int chunk = (D == 3) ? (int)blockIdx.y : ((D == 4) ? (int)blockIdx.z : 0);
-    grid_wait();
-    rows_tile<T, D, DYN, SCHEME, KIND>(P, R, C.sx, C.ty, C.nt, C.tz, blockIdx.x, i2, chunk, threadIdx.x,
+    rows_tile<T, D, DYN, SCHEME, KIND, true>(P, R, C.sx, C.ty, C.nt, C.tz, blockIdx.x, i2, chunk, threadIdx.x,
                                        reinterpret_cast<T*>(smem_raw));
 }
 
