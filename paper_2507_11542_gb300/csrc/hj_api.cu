@@ -379,10 +379,10 @@ std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtyp
 }
 
 // The launch shape for this grid: measured once per (shape, dtype, dynamics,
-// scheme, dissipation) over the model's best candidates (groups of
-// first-stage launches writing to a scratch buffer), then cached in the context. A tile override {ty, tz, occ, flags} (ty >= 1)
-// pins the rows and planes instead; it is validated once and cached like a
-// tuned shape.
+// scheme, dissipation) over the model's best candidates (groups of launches
+// writing to a scratch buffer), then cached in the context. A tile override
+// {ty, tz, occ, flags} (ty >= 1) pins the rows and planes instead; it is
+// validated once and cached like a tuned shape.
 hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_t* tile, RowsCfg* out) {
     const GridDev& G = P.g;
     std::vector<long long> key = {G.ndim, P.dynamics, P.scheme, dtype, G.n[0], G.n[1], G.n[2], G.n[3],
@@ -421,20 +421,22 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
         *out = it->second;
         return HJ_OK;
     }
-    std::vector<RowsCfg> cands = rows_candidates(ctx, P, dtype);
+    // two of a step's three stages read V^n as well, and their kernel may fit an
+    // SM fewer times than the first stage's: candidates are ranked and timed as
+    // such a stage (V^n = u)
+    StageParams T = P;
+    T.mode = kStage;
+    T.vn = T.u;
+    T.cv = 0.75;
+    T.cu = 0.25;
+    T.minv_after = 0;
+    std::vector<RowsCfg> cands = rows_candidates(ctx, T, dtype);
     if (cands.empty()) return fail(ctx, HJ_EINVAL, "no launch shape fits the row kernel");
     RowsCfg best = cands[0];
     if (cands.size() > 1) {
         const size_t bytes = (size_t)G.total * (dtype == HJ_F64 ? 8 : 4);
         hj_status st = ensure(ctx, &ctx->tune_buf, &ctx->tune_bytes, bytes);
         if (st) return st;
-        // timed as a first RK stage (reads u, writes the scratch buffer)
-        StageParams T = P;
-        T.mode = kStage;
-        T.vn = nullptr;
-        T.cv = 0.0;
-        T.cu = 1.0;
-        T.minv_after = 0;
         T.out = ctx->tune_buf;
         cudaEvent_t e0, e1;
         HJ_CUDA(ctx, cudaEventCreate(&e0));
