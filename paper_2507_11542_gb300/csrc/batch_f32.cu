@@ -19,14 +19,15 @@ cudaError_t launch_batch_stage_f32(const BatchTile* tiles, int ntiles, const Bat
 // After stage 3 of a step: count the step, and set up the next one. Every
 // step uses dt_full except the one that completes a slice, which is clipped
 // to land on the slice time (Listing 6) and also writes the slice output.
-// Only instances of lanes lane_lo .. lane_hi took this step (the lane is
-// tested first: other lanes' descriptors may be advancing concurrently).
-__global__ void batch_advance_kernel(BatchInst* insts, int n, int lane_lo, int lane_hi) {
+// One thread a tile: an instance's first tile advances it (other chains'
+// descriptors may be advancing concurrently).
+__global__ void batch_advance_kernel(const BatchTile* tiles, int ntiles, BatchInst* insts) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     grid_wait();
-    if (i >= n) return;
-    BatchInst& I = insts[i];
-    if (I.lane < lane_lo || I.lane > lane_hi) return;
+    if (i >= ntiles) return;
+    const BatchTile t = tiles[i];
+    if (t.tile != 0 || t.i2 != 0 || t.chunk != 0) return;
+    BatchInst& I = insts[t.inst];
     if (I.k >= I.steps_total) return;
     const int k = ++I.k;
     I.slice_out = nullptr;
@@ -42,8 +43,8 @@ __global__ void batch_advance_kernel(BatchInst* insts, int n, int lane_lo, int l
     }
 }
 
-cudaError_t launch_batch_advance(BatchInst* insts, int n, int lane_lo, int lane_hi, cudaStream_t s) {
-    return launch_dependent(batch_advance_kernel, dim3((n + 127) / 128), dim3(128), 0, s, insts, n, lane_lo, lane_hi);
+cudaError_t launch_batch_advance(const BatchTile* tiles, int ntiles, BatchInst* insts, cudaStream_t s) {
+    return launch_dependent(batch_advance_kernel, dim3((ntiles + 127) / 128), dim3(128), 0, s, tiles, ntiles, insts);
 }
 
 }  // namespace hj

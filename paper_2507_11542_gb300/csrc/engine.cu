@@ -90,6 +90,10 @@ void Engine::shutdown() {
     groups_.clear();
     if (cap_stream_) cudaStreamDestroy(cap_stream_);
     cap_stream_ = nullptr;
+    for (cudaStream_t c : chain_stream_) cudaStreamDestroy(c);
+    chain_stream_.clear();
+    if (cap_ev_) cudaEventDestroy(cap_ev_);
+    cap_ev_ = nullptr;
     cudaFree(arena_mem_);
     cudaFree(d_insts_);
     cudaFree(d_words_);
@@ -110,6 +114,7 @@ hj_status Engine::init(hj_ctx* ctx, cudaStream_t stream, int max_slots, size_t a
     HJ_CUDA(ctx, cudaMemsetAsync(d_insts_, 0, sizeof(BatchInst) * max_slots_, stream_));
     HJ_CUDA(ctx, cudaMalloc(&d_words_, 16 * (size_t)max_slots_));
     HJ_CUDA(ctx, cudaStreamCreateWithFlags(&cap_stream_, cudaStreamNonBlocking));
+    HJ_CUDA(ctx, cudaEventCreateWithFlags(&cap_ev_, cudaEventDisableTiming));
     if (multirate_) {
         HJ_CUDA(ctx, cudaEventCreateWithFlags(&fork_ev_, cudaEventDisableTiming));
         for (int l = 0; l < kLanes; ++l) {
@@ -326,7 +331,6 @@ hj_status Engine::activate(std::vector<int>* failed) {
         }
         D.dt_f = (float)D.dt;
         S.lane = !multirate_ ? 0 : lane_of(S.N);
-        D.lane = S.lane;
         // group
         const int dyn = S.prob.method.dynamics;
         const int scheme = S.prob.method.scheme;
@@ -510,21 +514,33 @@ hj_status Engine::rebuild_tiles() {
     for (size_t gi = 0; gi < groups_.size(); ++gi) {
         Group& g = groups_[gi];
         g.tiles.clear();
-        // by lane (the tiles of lanes >= l are a suffix), then largest instances
-        // first: their many tiles start early, small ones fill the tail
+        // largest instances first: their many tiles start early, small ones fill the tail
         std::vector<int> order;
         for (int i = 0; i < max_slots_; ++i)
             if (slots[i].used && slots[i].active && slots[i].group == (int)gi) order.push_back(i);
-        std::sort(order.begin(), order.end(), [&](int a, int b) {
-            return slots[a].lane != slots[b].lane ? slots[a].lane < slots[b].lane : slots[a].N > slots[b].N;
-        });
+        std::sort(order.begin(), order.end(), [&](int a, int b) { return slots[a].N > slots[b].N; });
         g.smem = 0;
-        for (int l = 0; l < kLanes; ++l) g.lane_off[l] = 0;
-        for (int i : order) {
-            append_tiles(slots[i], i, &g.tiles);
-            // tiles of lanes above this instance's start after it
-            for (int l = slots[i].lane + 1; l < kLanes; ++l) g.lane_off[l] = g.tiles.size();
-            g.smem = std::max(g.smem, rows_smem(slots[i].sx, slots[i].es));
+        for (int l = 0; l < kLanes; ++l) {
+            g.chains[l].clear();
+            std::vector<int> part[kChains];
+            long long load[kChains] = {};
+            for (int i : order) {
+                if (slots[i].lane != l) continue;
+                const int c = (int)(std::min_element(load, load + kChains) - load);
+                part[c].push_back(i);
+                load[c] += tiles_of(slots[i]);
+            }
+            for (const std::vector<int>& p : part) {
+                if (p.empty()) continue;
+                Chain c;
+                c.off = g.tiles.size();
+                for (int i : p) {
+                    append_tiles(slots[i], i, &g.tiles);
+                    g.smem = std::max(g.smem, rows_smem(slots[i].sx, slots[i].es));
+                }
+                c.end = g.tiles.size();
+                g.chains[l].push_back(c);
+            }
         }
         tiles_total_ += (long long)g.tiles.size();
         if (g.tiles.empty()) continue;
@@ -544,29 +560,50 @@ hj_status Engine::rebuild_tiles() {
     return HJ_OK;
 }
 
-// One RK3 step of the instances of lane `lane` and above.
-cudaError_t Engine::enqueue_step(cudaStream_t s, bool count, int lane, bool exact) {
-    for (int stage = 1; stage <= 3; ++stage)
-        for (const Group& g : groups_) {
-            const size_t off = g.lane_off[lane];
-            const size_t end = exact ? lane_end(g, lane) : g.tiles.size();
-            if (end <= off) continue;
-            const int nt = (int)(end - off);
-            cudaError_t e = g.dtype == HJ_F64 ? launch_batch_stage_f64(g.d_tiles + off, nt, d_insts_, stage, g.ndim,
-                                                                       g.dyn, g.scheme, g.threads, g.smem, s)
-                                              : launch_batch_stage_f32(g.d_tiles + off, nt, d_insts_, stage, g.ndim,
-                                                                       g.dyn, g.scheme, g.threads, g.smem, s);
-            if (e != cudaSuccess) return e;
-            if (count) {
-                launches += 1;
-                ctx_->launches += 1;
-            }
-        }
-    if (count) {
-        launches += 1;
-        ctx_->launches += 1;
+cudaError_t Engine::enqueue_step(const Group& g, const Chain& c, cudaStream_t s) {
+    const BatchTile* tiles = g.d_tiles + c.off;
+    const int nt = (int)(c.end - c.off);
+    for (int stage = 1; stage <= 3; ++stage) {
+        cudaError_t e = g.dtype == HJ_F64 ? launch_batch_stage_f64(tiles, nt, d_insts_, stage, g.ndim, g.dyn, g.scheme,
+                                                                   g.threads, g.smem, s)
+                                          : launch_batch_stage_f32(tiles, nt, d_insts_, stage, g.ndim, g.dyn, g.scheme,
+                                                                   g.threads, g.smem, s);
+        if (e != cudaSuccess) return e;
     }
-    return launch_batch_advance(d_insts_, max_slots_, lane, exact ? lane : kLanes - 1, s);
+    return launch_batch_advance(tiles, nt, d_insts_, s);
+}
+
+cudaError_t Engine::capture_lane(int lane, int K, cudaGraph_t* graph) {
+    cudaError_t e = cudaStreamBeginCapture(cap_stream_, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    e = cudaEventRecord(cap_ev_, cap_stream_);
+    std::vector<cudaStream_t> used;
+    size_t n = 0;
+    for (const Group& g : groups_)
+        for (const Chain& c : g.chains[lane]) {
+            cudaStream_t s = cap_stream_;
+            if (n > 0) {
+                if (e == cudaSuccess && chain_stream_.size() < n) {
+                    cudaStream_t fresh = nullptr;
+                    e = cudaStreamCreateWithFlags(&fresh, cudaStreamNonBlocking);
+                    if (e == cudaSuccess) chain_stream_.push_back(fresh);
+                }
+                if (e == cudaSuccess) {
+                    s = chain_stream_[n - 1];
+                    e = cudaStreamWaitEvent(s, cap_ev_, 0);
+                    if (e == cudaSuccess) used.push_back(s);
+                }
+            }
+            for (int k = 0; k < K && e == cudaSuccess; ++k) e = enqueue_step(g, c, s);
+            ++n;
+        }
+    for (cudaStream_t s : used) {  // (after an error too: a capture ends with its streams joined)
+        cudaError_t e2 = cudaEventRecord(cap_ev_, s);
+        if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(cap_stream_, cap_ev_, 0);
+        if (e == cudaSuccess) e = e2;
+    }
+    const cudaError_t e2 = cudaStreamEndCapture(cap_stream_, graph);
+    return e == cudaSuccess ? e2 : e;
 }
 
 long long Engine::dead_tiles() const {
@@ -605,40 +642,28 @@ hj_status Engine::run(int K) {
     // all lanes forked from stream_ and joined back into it.
     if (multirate_) e = cudaEventRecord(fork_ev_, stream_);
     for (int l = 0; l < (multirate_ ? kLanes : 1) && e == cudaSuccess; ++l) {
-        bool any = false;
-        long long per_step = 1;
-        for (const Group& g : groups_)
-            if ((multirate_ ? lane_end(g, l) : g.tiles.size()) > g.lane_off[l]) {
-                any = true;
-                per_step += 3;
-            }
-        if (!any) continue;
+        long long per_step = 0;
+        for (const Group& g : groups_) per_step += 4 * (long long)g.chains[l].size();
+        if (!per_step) continue;
         const int Kl = multirate_ ? kLaneMult[l] * K : K;
         cudaStream_t s = multirate_ ? lane_stream_[l] : stream_;
         if (multirate_) e = cudaStreamWaitEvent(s, fork_ev_, 0);
-        if (e == cudaSuccess && Kl >= 2) {
-            if (!exec_[l] || exec_K_[l] != Kl) {
-                if (exec_[l]) {
-                    cudaStreamSynchronize(stream_);
-                    cudaGraphExecDestroy(exec_[l]);
-                    exec_[l] = nullptr;
-                }
-                cudaGraph_t graph = nullptr;
-                e = cudaStreamBeginCapture(cap_stream_, cudaStreamCaptureModeThreadLocal);
-                for (int k = 0; k < Kl && e == cudaSuccess; ++k) e = enqueue_step(cap_stream_, false, l, multirate_);
-                cudaError_t e2 = cudaStreamEndCapture(cap_stream_, &graph);
-                if (e == cudaSuccess) e = e2;
-                if (e == cudaSuccess) e = cudaGraphInstantiate(&exec_[l], graph, 0);
-                if (graph) cudaGraphDestroy(graph);
-                exec_K_[l] = Kl;
+        if (e == cudaSuccess && (!exec_[l] || exec_K_[l] != Kl)) {
+            if (exec_[l]) {
+                cudaStreamSynchronize(stream_);
+                cudaGraphExecDestroy(exec_[l]);
+                exec_[l] = nullptr;
             }
-            if (e == cudaSuccess) e = cudaGraphLaunch(exec_[l], s);
-            if (e == cudaSuccess) {
-                launches += per_step * Kl;
-                ctx_->launches += per_step * Kl;
-            }
-        } else {
-            for (int k = 0; k < Kl && e == cudaSuccess; ++k) e = enqueue_step(s, true, l, multirate_);
+            cudaGraph_t graph = nullptr;
+            e = capture_lane(l, Kl, &graph);
+            if (e == cudaSuccess) e = cudaGraphInstantiate(&exec_[l], graph, 0);
+            if (graph) cudaGraphDestroy(graph);
+            exec_K_[l] = Kl;
+        }
+        if (e == cudaSuccess) e = cudaGraphLaunch(exec_[l], s);
+        if (e == cudaSuccess) {
+            launches += per_step * Kl;
+            ctx_->launches += per_step * Kl;
         }
         if (multirate_ && e == cudaSuccess) e = cudaEventRecord(lane_ev_[l], s);
         if (multirate_ && e == cudaSuccess) e = cudaStreamWaitEvent(stream_, lane_ev_[l], 0);

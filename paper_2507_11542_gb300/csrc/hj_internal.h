@@ -255,15 +255,14 @@ struct BatchInst {
     void* out;                // slice outputs: n_slices x nodes elements
     long long nodes;
     int elem;                 // element size in bytes
-    int lane;                 // rate class: advanced by the step graphs of lanes 0 .. lane
 };
 
 cudaError_t launch_batch_stage_f32(const BatchTile* tiles, int ntiles, const BatchInst* insts, int stage, int ndim,
                                    int dynamics, int scheme, int threads, size_t smem, cudaStream_t s);
 cudaError_t launch_batch_stage_f64(const BatchTile* tiles, int ntiles, const BatchInst* insts, int stage, int ndim,
                                    int dynamics, int scheme, int threads, size_t smem, cudaStream_t s);
-// Advances the instances of lanes lane_lo .. lane_hi (BatchInst::lane).
-cudaError_t launch_batch_advance(BatchInst* insts, int n, int lane_lo, int lane_hi, cudaStream_t s);
+// Advances the instances of these tiles.
+cudaError_t launch_batch_advance(const BatchTile* tiles, int ntiles, BatchInst* insts, cudaStream_t s);
 
 // max over nodes of sum_d alpha_d(x)/dx_d, as the FP64 bit pattern, atomically
 // max-ed into *acc (which the caller zeroes first).

@@ -74,6 +74,25 @@ def test_batch_equals_each_solve_alone(ctx, dtype):
             assert rel_err(to_host(outs[k][s], spec.n), to_host(alone[s], spec.n)) <= tol, (k, s)
 
 
+@pytest.mark.parametrize("count", [1, 2, 3, 5])
+def test_chains_of_one_kind_equal_each_solve_alone(ctx, count):
+    """Members of one kind are split into concurrent chains of launches; they
+    end at different steps (several blocks of steps) and fill slices on the way."""
+    from paper_2507_11542_gb300 import solver
+    cases = []
+    for k in range(count):
+        g, V0 = W.double_integrator(31 + 17 * k, 0.5)
+        cases.append((g, lib_method(dynamics=DI), V0, [0.1, 0.3 + 0.2 * ((3 * k) % 5)]))
+    outs, times, stats = solver.solve_batch(ctx, [c[0] for c in cases], [c[1] for c in cases],
+                                            [to_dev(c[2]) for c in cases], [c[3] for c in cases])
+    for k, (g, m, V0, ts) in enumerate(cases):
+        alone, t_alone, st_alone = solver.solve(ctx, g, m, to_dev(V0), ts)
+        assert stats[k]["steps"] == st_alone["steps"], k
+        np.testing.assert_array_equal(times[k], t_alone)
+        for s in range(len(ts)):  # the 2-D solve alone may take the plane kernel
+            assert rel_err(to_host(outs[k][s], g.n), to_host(alone[s], g.n)) <= 1e-13, (k, s)
+
+
 def test_batch_fp64_matches_oracle(ctx):
     from paper_2507_11542_gb300 import solver
     cases = _mixed("float64")
