@@ -172,9 +172,9 @@ inline int rows_segment(int n0, int ty, int node_threads) {
 }
 // Edge threads beside a tile's node threads (the tile's last interfaces, one per
 // two columns and per row pair, and the halos). A block waits for its edge warps
-// in every plane: with one column of halo a thread the FP32 stage of 101^3 takes
+// in every plane: with one column of halo a thread the FP32 stage of 101^3 took
 // 15.6 us, with two (and half the threads) 21; in FP64, whose planes take longer,
-// 240 and 231 us.
+// 240 and 231 us (now 14.4 and 206).
 __host__ __device__ constexpr int rows_edge_cols(bool f64) { return f64 ? 2 : 1; }
 inline int rows_edge_threads(int sx, bool f64) {
     const int need = f64 ? (sx + 1) / 2 + 4 : sx + 4;

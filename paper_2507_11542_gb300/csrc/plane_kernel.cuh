@@ -2,15 +2,17 @@
 // mostly idle: one interface per thread, then one node per thread.
 //
 // An FP64 2-D stage of 101^2 nodes is one short chain of dependent operations per
-// thread, and with two rows a thread (rows_kernel.cuh) a chain of 11.4 us: one warp's FP64 instructions follow each other in 64 cycles each on its
-// quarter of the SM, while the other quarters have no warp. Here the
-// interfaces along both dimensions of a small tile are dealt out to the
-// threads of a block (FP32: two rows' or two gaps' at a time, packed as in the
-// row kernel), both halves go through shared memory, and each node is updated
-// by a thread of its own: 6.2 us (5 x 12 nodes a block, two blocks an SM), 44 us
-// instead of 50 on 511^2. FP32, whose stage is launch latency up to 301^2 (2.5 to
-// 2.8 us with either kernel), keeps the row kernel where that is faster: the
-// launch-shape tuner times both.
+// thread, and with two rows a thread (rows_kernel.cuh) a chain of 11.4 us: one
+// warp's FP64 instructions follow each other in 64 cycles each on its quarter of
+// the SM, while the other quarters have no warp. Here the interfaces along both
+// dimensions of a small tile are dealt out to the threads of a block (FP32: two
+// rows' or two gaps' at a time, packed as in the row kernel), both halves go
+// through shared memory, and each node is updated by a thread of its own: 6.2 us
+// (5 x 12 nodes a block, two blocks an SM), 44 us instead of 50 on 511^2; a whole
+// solve of 101^2 then took 2592 us, with the smoothness sums in integers 2438, and
+// with indices and cells ready before the wait for the kernel in front 2275. FP32,
+// whose stage is launch latency up to 301^2 (2.5 to 2.8 us with either kernel),
+// keeps the row kernel where that is faster: the launch-shape tuner times both.
 // Both evaluate an interface and a node with the same functions, so that the
 // results are the same bits.
 #pragma once
@@ -44,42 +46,81 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_kernel(const StagePara
     T* const ym = yp + (C.ty + 2) * C.sx;
     const T fl0 = SP<T>::floor(P, 0), fl1 = SP<T>::floor(P, 1);
 
-    grid_wait();
-    const T* __restrict__ u = R.u;
-    // V^n of this thread's (first) node, ahead of its use
-    T old = T(0);
-    const int x_own = t % C.sx, r_own = t / C.sx;
-    const bool own = x_own < sx && r_own < rv;
-    if (KIND == kKindCombine && own) old = ld(R.vn + (y0 + r_own) * nx + x0 + x_own);
-
-    // value at offset i of a line (n nodes from base, stride s), ghosts included
-    auto at = [&](int base, int i, int n, int s, bool periodic) -> T {
-        if (i >= 0 && i < n) return ld(u + base + i * s);
-        if (periodic) return ld(u + base + (i + (i < 0 ? n : -n)) * s);
-        const int e = i < 0 ? 0 : n - 1, inner = i < 0 ? 1 : n - 2;
-        return ghost_value(ld(u + base + e * s), ld(u + base + inner * s), i < 0 ? -i : i - (n - 1), g.extrap);
+    // One cell of the tile: where it goes, and its source or, of a ghost cell, the
+    // two outermost values and its distance from them.
+    struct Cell {
+        int to, a, b, m;  // to < 0: none; b < 0: no ghost cell
     };
-    for (int c = t; c < (rv + 6) * (sx + 6); c += C.nt) {
+    auto make_cell = [&](int c) {
+        Cell q{-1, 0, -1, 0};
         const int r = c / (sx + 6) - 3, x = c - (r + 3) * (sx + 6) - 3;
         const bool in_x = x >= 0 && x < sx, in_y = r >= 0 && r < rv;
-        if (in_y) V[(r + 3) * W + x + 3] = at((y0 + r) * nx, x0 + x, nx, 1, per0);
-        else if (in_x) V[(r + 3) * W + x + 3] = at(x0 + x, y0 + r, ny, nx, per1);
+        if (r >= rv + 3 || !(in_x || in_y)) return q;
+        q.to = (r + 3) * W + x + 3;
+        const int n = in_y ? nx : ny, s = in_y ? 1 : nx, base = in_y ? (y0 + r) * nx : x0 + x;
+        int i = in_y ? x0 + x : y0 + r;
+        if (in_y ? per0 : per1) i += i < 0 ? n : i >= n ? -n : 0;
+        if (i >= 0 && i < n) {
+            q.a = base + i * s;
+        } else {
+            q.a = base + (i < 0 ? 0 : n - 1) * s;
+            q.b = base + (i < 0 ? 1 : n - 2) * s;
+            q.m = i < 0 ? -i : i - (n - 1);
+        }
+        return q;
+    };
+    // One item of interfaces: its first row or gap, its column, and where its values begin.
+    const int n_x = (sx + 1) * ((rv + kW - 1) / kW), n_y = sx * ((rv + kW) / kW);
+    struct Item {
+        bool along_x;
+        int from, to;
+    };
+    auto make_item = [&](int i) {
+        Item q;
+        q.along_x = i < n_x;
+        const int k = q.along_x ? i : i - n_x, width = q.along_x ? sx + 1 : sx;
+        const int line = k / width, x = k - line * width;
+        q.from = q.along_x ? (line * kW + 3) * W + x : line * kW * W + x + 3;
+        q.to = line * kW * (q.along_x ? C.sx + 1 : C.sx) + x;
+        return q;
+    };
+
+    // A stage is a chain of latencies: what needs no values is done before the
+    // wait for the kernel in front (this thread's first cells, interface and node),
+    // and both cells are loaded before the first is used.
+    constexpr int kCells = 2;
+    Cell cell[kCells];
+#pragma unroll
+    for (int k = 0; k < kCells; ++k) cell[k] = make_cell(t + k * C.nt);
+    Item item = make_item(t);
+    const int r_own = t / C.sx, x_own = t - r_own * C.sx;
+    const bool own = x_own < sx && r_own < rv;
+
+    grid_wait();
+    const T* __restrict__ u = R.u;
+    T va[kCells], vb[kCells];
+#pragma unroll
+    for (int k = 0; k < kCells; ++k) {
+        va[k] = vb[k] = T(0);
+        if (cell[k].to >= 0) va[k] = ld(u + cell[k].a);
+        if (cell[k].b >= 0) vb[k] = ld(u + cell[k].b);
+    }
+    // V^n of this thread's (first) node, ahead of its use
+    T old = T(0);
+    if (KIND == kKindCombine && own) old = ld(R.vn + (y0 + r_own) * nx + x0 + x_own);
+#pragma unroll
+    for (int k = 0; k < kCells; ++k)
+        if (cell[k].to >= 0) V[cell[k].to] = cell[k].b >= 0 ? ghost_value(va[k], vb[k], cell[k].m, g.extrap) : va[k];
+    for (int c = t + kCells * C.nt; c < (rv + 6) * (sx + 6); c += C.nt) {
+        const Cell q = make_cell(c);
+        if (q.to >= 0) V[q.to] = q.b >= 0 ? ghost_value(ld(u + q.a), ld(u + q.b), q.m, g.extrap) : ld(u + q.a);
     }
     __syncthreads();
 
-    const int n_x = (sx + 1) * ((rv + kW - 1) / kW), n_y = sx * ((rv + kW) / kW);
     for (int i = t; i < n_x + n_y; i += C.nt) {
-        const bool along_x = i < n_x;
-        int line, x;  // first row, or first gap, and column
-        if (along_x) {
-            line = i / (sx + 1);
-            x = i - line * (sx + 1);
-        } else {
-            line = (i - n_x) / sx;
-            x = i - n_x - line * sx;
-        }
-        line *= kW;
-        const T* w0 = along_x ? V + (line + 3) * W + x : V + line * W + x + 3;
+        if (i != t) item = make_item(i);
+        const bool along_x = item.along_x;
+        const T* w0 = V + item.from;
         const int step = along_x ? 1 : W;
         T v[kW][6], pp[kW], pm[kW];
 #pragma unroll
@@ -89,7 +130,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_kernel(const StagePara
         iface_item<SCHEME>(v, along_x ? fl0 : fl1, pp, pm);
 #pragma unroll
         for (int l = 0; l < kW; ++l) {
-            const int o = along_x ? (line + l) * (C.sx + 1) + x : (line + l) * C.sx + x;
+            const int o = item.to + l * (along_x ? C.sx + 1 : C.sx);
             (along_x ? xp : yp)[o] = pp[l];
             (along_x ? xm : ym)[o] = pm[l];
         }
@@ -105,7 +146,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_kernel(const StagePara
 #pragma unroll
     for (int k = 0; k < 8; ++k) par[k] = SP<T>::param(P, k);
     for (int i = t; i < C.sx * rv; i += C.nt) {
-        const int r = i / C.sx, x = i - r * C.sx;
+        const int r = i == t ? r_own : i / C.sx, x = i - r * C.sx;
         if (x >= sx) continue;
         const int flat = (y0 + r) * nx + x0 + x;
         if (KIND == kKindCombine && i != t) old = ld(R.vn + flat);

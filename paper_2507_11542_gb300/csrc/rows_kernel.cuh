@@ -35,8 +35,9 @@ namespace hj {
 
 // Launch bounds, i.e. registers a thread (blocks have at most rows_max_threads).
 // FP32 stage of 101^3 / 161x113x79 at 640, 768, 896, 1024 threads (96, 80, 72, 64
-// registers): 16.7, 16.1, 15.7, 16.2 / 22.6, 20.5, 20.0, 20.7 us; of 81^4 at 768 and
-// 896: 0.69 and 0.71 ms.
+// registers): 16.7, 16.1, 15.7, 16.2 / 22.6, 20.5, 20.0, 20.7 us (now 14.4 / 18.5 at
+// 896); of 81^4 at 768 and 896: 0.69 and 0.71 ms, and with the lines of dimension 2
+// loaded a phase ahead 0.66 at 896 (now 0.636).
 template <typename T, int D> struct RowsBounds { static constexpr int kThreads = D == 2 ? 768 : 896; };
 template <int D> struct RowsBounds<double, D> { static constexpr int kThreads = kRowsThreadsF64; };
 
@@ -172,8 +173,10 @@ __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __rest
     // -3, -2, -1 or sx, sx+1, sx+2 of a row. Sources do not change from plane to
     // plane. Ghost cells (extrapolated edges) need the two outermost values at
     // their end of the line, which are loaded one plane before they are made. In a
-    // launch of one wave the blocks that make them take the longest: this path is
-    // kept short.
+    // launch of one wave the blocks that make them take the longest, and this path
+    // is kept short: without any edge work a 161x113x79 FP32 stage takes 15.7 us of
+    // 19.0, and whole lines in place of sides (eight row threads with twelve cells
+    // more than the others) cost 0.8 us.
     constexpr int kCols = rows_edge_cols(sizeof(T) == 8);
     struct Side {
         int src[3];  // flat index, or -1: a ghost cell
@@ -266,7 +269,9 @@ __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __rest
         if (row_job) ghosts(row, row_to + o, kP, row_high ? T(1) : T(-1));
     };
 
-    // first two planes: all copies and all sources are under way before the first ghost cell waits for its own
+    // first two planes: all copies and all sources are under way before the first
+    // ghost cell waits for its own (the stages of 161x113x79 and 101^3 in FP32 took
+    // 19.0 and 15.0 us with one plane's sources after the other, 18.5 and 14.4 so)
     if constexpr (WAIT) grid_wait();
     const bool second = C.zbeg + 1 < C.zend;
     Side first[2 * kCols + 1], next[2 * kCols + 1];
