@@ -441,10 +441,14 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
         cudaEvent_t e0, e1;
         HJ_CUDA(ctx, cudaEventCreate(&e0));
         HJ_CUDA(ctx, cudaEventCreate(&e1));
-        // launches of less than about 100 us are timed in groups: the event
-        // clock advances in steps of about two microseconds
+        // Short launches are timed in rows of up to eight, as a step or a solve runs
+        // them: the event clock advances in steps of about two microseconds, and of
+        // a row only the first launch finds an empty chip. Where two blocks fit an
+        // SM, the next launch's blocks wait beside the running ones wherever there
+        // is room, some SMs get two of them and others none (103 x 47 x 44 FP64
+        // ENO3: a shape at 52 us a launch in pairs took 88 in a step; now 55 to 57).
         const double per_us = dtype == HJ_F64 ? 4e3 : 4e4;  // nodes a microsecond, roughly
-        const int group = (int)std::min(8.0, std::max(1.0, std::ceil(100.0 * per_us / (double)G.total)));
+        const int group = (int)std::min(8.0, std::max(1.0, std::ceil(600.0 * per_us / (double)G.total)));
         const auto timed = [&](const RowsCfg& c, int reps, float* ms_min) -> cudaError_t {
             cudaError_t e = cudaSuccess;
             for (int rep = 0; rep < reps && e == cudaSuccess; ++rep) {
@@ -458,7 +462,7 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
             }
             return e;
         };
-        // about a millisecond of launches first (an idle GPU's clocks rise meanwhile), every candidate twice,
+        // about a millisecond of launches first (an idle GPU's clocks rise meanwhile), every candidate once or twice,
         // then the five best again: a pick by one disturbed group cost up to a third of a step
         cudaError_t e = cudaSuccess;
         const int warm = (int)std::min(64.0, std::max(1.0, 1000.0 * per_us / (double)G.total));
@@ -467,7 +471,7 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
         for (size_t i = 0; i < cands.size() && e == cudaSuccess; ++i) {
             e = rows_launch(ctx, T, cands[i], dtype);  // loads the kernel, fills the caches
             float ms = 1e30f;
-            if (e == cudaSuccess) e = timed(cands[i], 2, &ms);
+            if (e == cudaSuccess) e = timed(cands[i], group >= 4 ? 1 : 2, &ms);
             took.push_back({ms, i});
         }
         std::sort(took.begin(), took.end());
