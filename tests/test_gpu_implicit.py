@@ -39,6 +39,21 @@ def test_surface_matches_oracle(ctx, shape, periodic, dtype):
     assert np.max(np.abs(got - ref)) <= tol * scale
 
 
+@pytest.mark.parametrize("n", [(4, 5), (33, 300), (129, 7), (160, 131), (261, 257)])
+@pytest.mark.parametrize("dtype", ["float64", "float32"])
+def test_surface_rows_and_threads_of_a_block(ctx, n, dtype):
+    """The rows a block covers and its threads along a row follow the grid: odd
+    remainders of both. Bounds as above (unit roundoff times the terms of a sum)."""
+    from paper_2507_11542_gb300 import solver
+    g = W.GridSpec(n, (-1.2, -1.0), (1.1, 1.3))
+    shapes = [{"kind": I.SPHERE, "center": (0.2, -0.3), "radius": 0.7},
+              {"kind": I.RECTANGLE, "op": I.UNION, "center": (-0.4, 0.5), "axes": (0.3, 0.6)}]
+    got = to_host(solver.implicit_surface(ctx, g, shapes, dtype), g.n)
+    ref = I.implicit_surface(g, shapes)
+    tol = 1e-14 if dtype == "float64" else 1e-6
+    assert np.max(np.abs(got - ref)) <= tol * float(np.max(np.abs(ref)))
+
+
 def test_surface_2d_and_4d_and_host_output(ctx):
     from paper_2507_11542_gb300 import _lib as L
     g2 = W.GridSpec((51, 33), (-1.0, -1.0), (1.0, 1.0))
