@@ -96,10 +96,17 @@ __device__ __forceinline__ T stage_value(const StageParams& P, const StageRun<T>
     const T w = fma_rn(R.dt, yd, center);
     if constexpr (KIND != kKindCombine) return w;
     // cv V^n + cu w; with cv + cu = 1 FP32 takes it as w + cv (V^n - w): the
-    // difference is small, so that one rounding alone counts
+    // difference is small, so that one rounding alone counts. Where it is not
+    // finite (an infinite value on either side, or two of opposite sign near the
+    // largest) the sum as it stands keeps what is infinite infinite.
     T res;
-    if constexpr (std::is_same<T, double>::value) res = fma_rn(R.cu, w, mul_rn(R.cv, old));
-    else res = fma_rn(R.cv, add_rn(old, -w), w);
+    if constexpr (std::is_same<T, double>::value) {
+        res = fma_rn(R.cu, w, mul_rn(R.cv, old));
+    } else {
+        const T diff = add_rn(old, -w);
+        res = fma_rn(R.cv, diff, w);
+        if (!(fabsf(diff) <= 3.402823466e38f)) res = fma_rn(R.cu, w, mul_rn(R.cv, old));
+    }
     return R.minv ? fmin(res, old) : res;
 }
 
