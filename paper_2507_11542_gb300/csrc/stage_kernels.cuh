@@ -70,6 +70,36 @@ __device__ __forceinline__ double over_dx(double raw, double dx, double inv_dx) 
     return (__double2hiint(q) & 0x7ff00000) == 0x7ff00000 ? q : c;
 }
 
+// FP32 WENO5 of two lines' interfaces (values v) over the whole range of FP32: a
+// line whose largest difference is 2 or more has all five scaled by the power of
+// two that brings it to [1, 2), and `unit` is what its results then count in.
+// Unscaled, the squared smoothness sums leave FP32 from differences of about 3e8
+// on. Where they do not the results are the same bits (the epsilon's floor is far
+// below the last place of the rest from differences of 1 on).
+__device__ __forceinline__ void weno5_lines(const float (&v)[2][6], float* pp, float* pm, float* unit) {
+    float e[2][5], by[2];
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        float top = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            e[l][k] = __fadd_rn(v[l][k + 1], -v[l][k]);
+            top = fmaxf(top, fabsf(e[l][k]));
+        }
+        const unsigned x = min(max(__float_as_uint(top) >> 23, 127u), 253u);  // 2^(x - 127) <= top, both powers normal
+        unit[l] = __uint_as_float(x << 23);
+        by[l] = __uint_as_float((254u - x) << 23);
+    }
+    F2 d[5], p, m;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) d[k] = lanes(__fmul_rn(e[0][k], by[0]), __fmul_rn(e[1][k], by[1]));
+    weno_iface2(d[0], d[1], d[2], d[3], d[4], p, m);
+    pp[0] = lane_a(p);
+    pp[1] = lane_b(p);
+    pm[0] = lane_a(m);
+    pm[1] = lane_b(m);
+}
+
 constexpr int kUpwindThreads = 128;
 constexpr int kUpwindRun = 8;
 
@@ -109,6 +139,7 @@ __global__ void __launch_bounds__(kUpwindThreads) upwind_kernel(const UpwindPara
         const T slope = (extrap == HJ_EXTRAP_LINEAR) ? (e - i) : fabs(e - i) * sgn(e);
         return add_rn(e, mul_rn(T(j < 0 ? -j : j - (n - 1)), slope));
     };
+    T unit[kLines];  // FP32 WENO5: of the last results (weno5_lines)
     auto store = [&](int j, const T* left, const T* right) {  // interface j: right = p+ of node j-1, left = p- of node j
 #pragma unroll
         for (int l = 0; l < kLines; ++l) {
@@ -116,6 +147,10 @@ __global__ void __launch_bounds__(kUpwindThreads) upwind_kernel(const UpwindPara
             if constexpr (SCHEME == HJ_WENO5) {
                 a *= inv_6dx;
                 b *= inv_6dx;
+                if constexpr (sizeof(T) == 4) {
+                    a *= unit[l];
+                    b *= unit[l];
+                }
             } else {
                 a = over_dx(a, dx, inv_dx);
                 b = over_dx(b, dx, inv_dx);
@@ -141,6 +176,7 @@ __global__ void __launch_bounds__(kUpwindThreads) upwind_kernel(const UpwindPara
             for (int l = 0; l < kLines; ++l) next[l] = at(base[l], j + 3);
         }
         if constexpr (std::is_same<T, double>::value && SCHEME == HJ_WENO5) walk.eval(floor, right[0], left[0]);
+        else if constexpr (SCHEME == HJ_WENO5) weno5_lines(v, right, left, unit);
         else iface_item<SCHEME>(v, floor, right, left);
         store(j, left, right);
         if (!more) break;
