@@ -771,8 +771,7 @@ hj_status hj_upwind(hj_ctx* ctx, const hj_grid* grid, const hj_method* method, i
     P.pp = pp;
     P.weno_floor = weno_floor(P.g, dtype, dim) * (dtype == HJ_F64 ? 12.0 : 1.0);
     P.dx = P.g.dx[dim];
-    P.inv_dx = P.g.inv_dx[dim];
-    P.inv_6dx = P.inv_dx / 6.0;
+    P.inv_6dx = P.g.inv_dx[dim] / 6.0;
     ctx->launches += 1;
     cudaError_t e = dtype == HJ_F64 ? launch_upwind_f64(P, method->scheme, ctx->stream)
                                     : launch_upwind_f32(P, method->scheme, ctx->stream);

@@ -140,7 +140,7 @@ struct UpwindParams {
     void* pm;
     void* pp;
     double weno_floor;  // FP64: times 12 (see StageParams)
-    double dx, inv_dx;
+    double dx;
     double inv_6dx;     // 1 / (6 dx)
 };
 

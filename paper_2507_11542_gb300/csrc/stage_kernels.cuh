@@ -60,15 +60,8 @@ __global__ void __launch_bounds__(kBX * kBY) stage_kernel(const StageParams P) {
 // a run of interfaces of one line (FP32: of two lines, one per lane), which in
 // FP64 WENO5 reuse their differences (Weno5Line: 15 FP64 instructions an
 // interface, where two one-sided evaluations per node took 50). 101^3 FP64, all
-// three dimensions: 318 -> 153 us, 136 with the sums u in integers.
-__device__ __forceinline__ float over_dx(float raw, float dx, float) { return raw / dx; }
-// raw / dx by the reciprocal and one Newton correction with the exact residual
-// (the correctly rounded quotient but for rare last bits); not finite: as it is.
-__device__ __forceinline__ double over_dx(double raw, double dx, double inv_dx) {
-    const double q = raw * inv_dx;
-    const double c = fma(fma(-q, dx, raw), inv_dx, q);
-    return (__double2hiint(q) & 0x7ff00000) == 0x7ff00000 ? q : c;
-}
+// three dimensions: 318 -> 153 us, 136 with the sums u in integers. The ENO schemes
+// work on divided differences, as their definition does (EnoLine).
 
 // FP32 WENO5 of two lines' interfaces (values v) over the whole range of FP32: a
 // line whose largest difference is 2 or more has all five scaled by the power of
@@ -114,16 +107,17 @@ __device__ __forceinline__ T line_node(const T* u, int j, int n, long long s, bo
     return add_rn(e, mul_rn(T(j < 0 ? -j : j - (n - 1)), slope));
 }
 
-// The derivatives from what an interface evaluation returns.
+// The derivatives from what an interface evaluation returns (WENO5: six times the
+// raw ones, in FP32 in units of weno5_lines; ENO: the derivatives).
 template <int SCHEME>
-__device__ __forceinline__ float derivative(float raw, float unit, const UpwindParams& P) {
-    if constexpr (SCHEME == HJ_WENO5) return raw * (float)P.inv_6dx * unit;
-    else return over_dx(raw, (float)P.dx, (float)P.inv_dx);
+__device__ __forceinline__ float derivative(float r, float unit, const UpwindParams& P) {
+    if constexpr (SCHEME == HJ_WENO5) return r * (float)P.inv_6dx * unit;
+    else return r;
 }
 template <int SCHEME>
-__device__ __forceinline__ double derivative(double raw, double, const UpwindParams& P) {
-    if constexpr (SCHEME == HJ_WENO5) return raw * P.inv_6dx;
-    else return over_dx(raw, P.dx, P.inv_dx);
+__device__ __forceinline__ double derivative(double r, double, const UpwindParams& P) {
+    if constexpr (SCHEME == HJ_WENO5) return r * P.inv_6dx;
+    else return r;
 }
 
 constexpr int kUpwindThreads = 128;
@@ -183,8 +177,17 @@ __global__ void __launch_bounds__(kUpwindThreads) upwind_row_kernel(const Upwind
             for (int k = kFrom; k < 6 - kFrom; ++k) v[l][k] = line_node(row, j[l] - 3 + k, n, 1LL, periodic, P.g.extrap);
         }
     }
-    if constexpr (SCHEME == HJ_WENO5) weno5_lines(v, right, left, unit);
-    else iface_item<SCHEME>(v, 0.0f, right, left);
+    if constexpr (SCHEME == HJ_WENO5) {
+        weno5_lines(v, right, left, unit);
+    } else {
+        const EnoSpacing<float> h((float)P.dx);
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+            EnoLine<float, SCHEME> e;
+            e.start(v[l], h);
+            e.eval(h, right[l], left[l]);
+        }
+    }
 #pragma unroll
     for (int l = 0; l < 2; ++l) {
         if (l == 1 && !two) break;
@@ -204,7 +207,8 @@ __global__ void __launch_bounds__(kUpwindThreads) upwind_kernel(const UpwindPara
     const T* __restrict__ u = static_cast<const T*>(P.u);
     T* __restrict__ pm = static_cast<T*>(P.pm);
     T* __restrict__ pp = static_cast<T*>(P.pp);
-    const T floor = T(P.weno_floor);
+    [[maybe_unused]] const T floor = T(P.weno_floor);
+    [[maybe_unused]] const EnoSpacing<T> h(T(P.dx));
     grid_wait();
     const long long item = (long long)blockIdx.x * kUpwindThreads + threadIdx.x;
     if (item >= group * runs) return;
@@ -232,9 +236,15 @@ __global__ void __launch_bounds__(kUpwindThreads) upwind_kernel(const UpwindPara
     for (int l = 0; l < kLines; ++l)
 #pragma unroll
         for (int k = 0; k < 6; ++k) v[l][k] = at(base[l], j0 - 3 + k);
+    constexpr bool kWeno64 = SCHEME == HJ_WENO5 && sizeof(T) == 8;
     [[maybe_unused]] Weno5Line walk;
-    if constexpr (std::is_same<T, double>::value && SCHEME == HJ_WENO5)
+    [[maybe_unused]] EnoLine<T, SCHEME> eno[kLines];
+    if constexpr (kWeno64) {
         walk.start(v[0][0], v[0][1], v[0][2], v[0][3], v[0][4], v[0][5]);
+    } else if constexpr (SCHEME != HJ_WENO5) {
+#pragma unroll
+        for (int l = 0; l < kLines; ++l) eno[l].start(v[l], h);
+    }
 #pragma unroll 1
     for (int j = j0;; ++j) {
         T left[kLines], right[kLines], next[kLines];
@@ -243,21 +253,29 @@ __global__ void __launch_bounds__(kUpwindThreads) upwind_kernel(const UpwindPara
 #pragma unroll
             for (int l = 0; l < kLines; ++l) next[l] = at(base[l], j + 3);
         }
-        if constexpr (std::is_same<T, double>::value && SCHEME == HJ_WENO5) walk.eval(floor, right[0], left[0]);
-        else if constexpr (SCHEME == HJ_WENO5) weno5_lines(v, right, left, unit);
-        else iface_item<SCHEME>(v, floor, right, left);
+        if constexpr (kWeno64) {
+            walk.eval(floor, right[0], left[0]);
+        } else if constexpr (SCHEME == HJ_WENO5) {
+            weno5_lines(v, right, left, unit);
+        } else {
+#pragma unroll
+            for (int l = 0; l < kLines; ++l) eno[l].eval(h, right[l], left[l]);
+        }
         store(j, left, right);
         if (!more) break;
-        if constexpr (std::is_same<T, double>::value && SCHEME == HJ_WENO5) {
+        if constexpr (kWeno64) {
             walk.slide(v[0][5], next[0]);
             v[0][5] = next[0];
-        } else {
+        } else if constexpr (SCHEME == HJ_WENO5) {
 #pragma unroll
             for (int l = 0; l < kLines; ++l) {
 #pragma unroll
                 for (int k = 0; k < 5; ++k) v[l][k] = v[l][k + 1];
                 v[l][5] = next[l];
             }
+        } else {
+#pragma unroll
+            for (int l = 0; l < kLines; ++l) eno[l].slide(next[l], h);
         }
     }
 }

@@ -1,6 +1,6 @@
 """hj_upwind beyond the parity fields: FP32 data of any size, FP32 lines of
 dimension 0 (interfaces dealt out two a thread, whatever the lines) at the sizes
-where the deal can go wrong, and what dimension 0 costs beside the others."""
+where the deal can go wrong, what dimension 0 costs beside the others, and ENO choices that are ties."""
 import numpy as np
 import pytest
 
@@ -80,3 +80,50 @@ def test_fp32_dimension_0_costs_what_the_others_do(ctx):
 
     best(2)
     assert best(0) <= 2.0 * best(2)
+
+
+@pytest.mark.parametrize("scheme", [2, 3])
+@pytest.mark.parametrize("dtype", ["float64", "float32"])
+def test_eno_choices_on_ties(ctx, scheme, dtype):
+    """A slope with a zigzag of one node on top: the two second differences to
+    choose from are equal and opposite but for rounding at every interface, and
+    either choice is the scheme's. hj_upwind forms the divided differences of the
+    definition, so that in FP64 it makes the oracle's choice even there (the other
+    one is a whole second difference away, most of the derivative here), and in
+    FP32 the choices of the same formulas in float32 (restated here)."""
+    from paper_2507_11542_gb300 import solver
+    spec = W.GridSpec((46, 38, 26), (-1.0, -1.3, -0.7), (1.0, 1.3, 0.7))
+    m_o, m = oracle_method(scheme=scheme, dynamics=NORM, extrap=1), lib_method(scheme=scheme, dynamics=NORM, extrap=1)
+    T = np.dtype(dtype).type
+    for dim in range(3):
+        r = np.random.default_rng(dim)
+        across = tuple(1 if k == dim else spec.n[k] for k in range(3))
+        i = np.arange(spec.n[dim]).reshape([-1 if k == dim else 1 for k in range(3)])
+        V = np.asfortranarray(r.uniform(-1.0, 1.0, across) * i * 0.03 + r.uniform(0.1, 1.0, across) * (-1.0) ** i)
+        pm, pp = solver.upwind(ctx, spec, m, to_dev(V, dtype), dim)
+        got_m, got_p = to_host(pm, spec.n), to_host(pp, spec.n)
+        if dtype == "float64":
+            want_m, want_p = O.upwind(spec, m_o, V, dim)
+            assert rel_err(got_m, want_m) <= 1e-12
+            assert rel_err(got_p, want_p) <= 1e-12
+            continue
+        # the definition in float32 on the nodes whose stencil needs no ghost cell
+        v = np.moveaxis(V.astype(np.float32), dim, 0)
+        n = spec.n[dim]
+        dx = T((spec.hi[dim] - spec.lo[dim]) / (n - 1))
+        d1 = (v[1:] - v[:-1]) / dx                      # d1[k]: between nodes k and k+1
+        d2 = (d1[1:] - d1[:-1]) / (T(2) * dx)           # d2[k]: node k+1
+        d3 = (d2[1:] - d2[:-1]) / (T(3) * dx)           # d3[k]: between nodes k+1 and k+2
+        k = np.arange(2, n - 3)                         # interfaces k + 1/2
+        left = np.abs(d2[k - 1]) <= np.abs(d2[k])
+        c = np.where(left, d2[k - 1], d2[k]).astype(np.float64)
+        h = float(dx)
+        right_m, left_p = d1[k].astype(np.float64) + c * h, d1[k].astype(np.float64) - c * h
+        if scheme == 3:
+            a, b = np.where(left, d3[k - 2], d3[k - 1]), np.where(left, d3[k - 1], d3[k])
+            cs = np.where(np.abs(a) <= np.abs(b), a, b).astype(np.float64)
+            right_m += cs * np.where(left, 2.0, -1.0) * h * h
+            left_p += cs * np.where(left, -1.0, 2.0) * h * h
+        # two or four more roundings of FP32
+        assert rel_err(np.moveaxis(got_m, dim, 0)[k + 1], right_m) <= 1e-6
+        assert rel_err(np.moveaxis(got_p, dim, 0)[k], left_p) <= 1e-6
