@@ -156,9 +156,12 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_kernel(const StagePara
         T xc[2] = {T(0), T(0)};
         if constexpr (uses_coord<2, DYN>(0)) xc[0] = coord(SP<T>::lo(P, 0), x0 + x, SP<T>::dx(P, 0));
         if constexpr (uses_coord<2, DYN>(1)) xc[1] = coord(SP<T>::lo(P, 1), y0 + r, SP<T>::dx(P, 1));
-        const T res = stage_value<T, 2, DYN, KIND>(P, R, par, xc, T(0), T(0), S, Q, hh, P.alpha_global,
-                                                         V[(r + 3) * W + x + 3], old);
-        R.out[flat] = res;
+        T res[1], w[1];
+        const T vn[1] = {old};
+        res[0] = stage_value<T, 2, DYN, KIND>(P, R, par, xc, T(0), T(0), S, Q, hh, P.alpha_global,
+                                              V[(r + 3) * W + x + 3], old, w[0]);
+        finish_values<T, 2, KIND>(R, res, w, vn);
+        R.out[flat] = res[0];
     }
 }
 
