@@ -19,7 +19,7 @@ template <typename T, int D, int DYN, int SCHEME, int KIND>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? kRowsThreadsF32 : kRowsThreadsF64, 1)
     batch_kernel(const BatchTile* tiles, const BatchInst* insts, const int stage) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    grid_wait();  // the descriptors change from step to step
+    grid_wait_only();  // the descriptors change from step to step
     const BatchTile t = tiles[blockIdx.x];
     const BatchInst& I = insts[t.inst];
     if (I.k >= I.steps_total) return;  // this instance has finished (block-uniform)

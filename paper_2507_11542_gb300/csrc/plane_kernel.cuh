@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_kernel(const StagePara
     const int r_own = t / C.sx, x_own = t - r_own * C.sx;
     const bool own = x_own < sx && r_own < rv;
 
-    grid_wait();
+    grid_wait_only();
     const T* __restrict__ u = R.u;
     T va[kCells], vb[kCells];
 #pragma unroll
@@ -116,6 +116,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_kernel(const StagePara
         if (q.to >= 0) V[q.to] = q.b >= 0 ? ghost_value(ld(u + q.a), ld(u + q.b), q.m, g.extrap) : ld(u + q.a);
     }
     __syncthreads();
+    grid_next();
 
     for (int i = t; i < n_x + n_y; i += C.nt) {
         if (i != t) item = make_item(i);

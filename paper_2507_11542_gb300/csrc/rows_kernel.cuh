@@ -296,7 +296,7 @@ __device__ __forceinline__ void edge_warps(const StageParams& P, const T* __rest
     // first two planes: all copies and all sources are under way before the first
     // ghost cell waits for its own (the stages of 161x113x79 and 101^3 in FP32 took
     // 19.0 and 15.0 us with one plane's sources after the other, 18.5 and 14.4 so)
-    if constexpr (WAIT) grid_wait();
+    if constexpr (WAIT) grid_wait_only();
     const bool second = C.zbeg + 1 < C.zend;
     Side first[2 * kCols + 1], next[2 * kCols + 1];
     copy_all(C.zbeg, 0);
@@ -421,7 +421,7 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
         xb[1] = coord(SP<T>::lo(P, 1), y1, SP<T>::dx(P, 1));
     }
     if constexpr (D == 4 && uses_coord<D, DYN>(2)) xa[2] = xb[2] = coord(SP<T>::lo(P, 2), C.i2, SP<T>::dx(P, 2));
-    if constexpr (WAIT) grid_wait();
+    if constexpr (WAIT) grid_wait_only();
     const T* __restrict__ trig = Trig<T>::get(P);       // cos of the dimension-2 coordinate
     const T* __restrict__ trig_s = uses_angle<D, DYN>() ? trig + g.n[2] : trig;  // sin
     T cos2 = T(0), sin2 = T(0);  // angle of dimension 2 (fixed for the block in 4-D, the next plane's in 3-D)
@@ -492,6 +492,7 @@ __device__ __forceinline__ void node_warps(const StageParams& P, const StageRun<
     put_own(smem, q[2]);
     if (D >= 3 && C.zbeg + 1 < C.zend) put_own(smem + buf, q[3]);
     block_barrier(C.nt);
+    grid_next();
 
 #pragma unroll 1
     for (int z = C.zbeg; z < C.zend; ++z) {
