@@ -324,11 +324,17 @@ cudaError_t rows_launch(hj_ctx* ctx, const StageParams& P0, const RowsCfg& c, in
     return dtype == HJ_F64 ? launch_rows_f64(P, c, ctx->stream) : launch_rows_f32(P, c, ctx->stream);
 }
 
-// Candidate shapes ranked by a simple cost model: the work of the busiest SM
-// (blocks x warps x planes, with a plane and a half of prologue per chunk), and
-// at least the latency of its waves one after the other. The twenty best are
-// timed.
-std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtype) {
+// Shapes of the row kernel ranked by a simple cost model, the cheapest first: the
+// work of the busiest SM (blocks x warps x planes, with some planes of prologue a
+// chunk), and at least the latency of its waves one after the other (a plane of a
+// wave lasts as long as some warps' work). quick: half a plane of prologue and
+// 6 warps in FP64, 22 in FP32; else one and a half planes and 10 warps. Over 32
+// grids of 2 to 4 dimensions, all shapes timed, the quick one's first is within 4 %
+// (FP64) and 6 % (FP32) of the best on average on grids of up to 1 M nodes (16 % at
+// most, the other's 55 %); on the largest (81^4) the other's twenty hold the best
+// within 1 %, the quick one's within 5 %, while on small ones they miss it by up to
+// 27 % (200 x 30 x 30 FP32).
+std::vector<RowsCfg> rows_ranked(const StageParams& P, int dtype, int sm_count, bool quick) {
     const GridDev& G = P.g;
     const int nx = G.n[0], ny = G.n[1];
     const int D = G.ndim;
@@ -336,6 +342,7 @@ std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtyp
     const bool f64 = dtype == HJ_F64;
     static const int tzs[] = {1, 2, 3, 4, 5, 6, 8, 10, 13, 16, 20, 24, 32, 48, 64, 128, 256};
     static const int node_threads[] = {32, 64, 96, 128, 192, 256, 384, 512};
+    const double prologue = quick ? 0.5 : 1.5, wave = !quick ? 10.0 : f64 ? 6.0 : 22.0, tail = quick ? 0.3 : 0.1;
     std::vector<std::pair<double, RowsCfg>> scored;
     for (int ty : {2, 3, 4, 5, 6, 7, 8}) {
         if (ty > ny && ty != 2) continue;
@@ -345,35 +352,46 @@ std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtyp
             const int sx = rows_segment(nx, ty, nn);
             if (sx == last_sx || (sx < 12 && sx < nx)) continue;
             last_sx = sx;
+            const int nt = rows_node_threads(sx, ty) + rows_edge_threads(sx, f64);
+            if (nt > rows_max_threads(f64)) continue;
+            const int bps = rows_bps(P, make_rows_cfg(G, sx, ty, 1, nt), dtype);  // (whatever the planes)
+            if (bps <= 0) continue;
             for (int k = 0; k < (D >= 3 ? (int)(sizeof tzs / sizeof tzs[0]) + 1 : 1); ++k) {
                 const int tz = D < 3 ? 1 : k < (int)(sizeof tzs / sizeof tzs[0]) ? tzs[k] : ns;
                 if (D >= 3 && tz >= ns && k < (int)(sizeof tzs / sizeof tzs[0])) continue;
-                const RowsCfg c = make_rows_cfg(G, sx, ty, tz, rows_node_threads(sx, ty) + rows_edge_threads(sx, dtype == HJ_F64));
-                if (c.nchunks > 65535 || c.nt > rows_max_threads(f64)) continue;
-                const int bps = rows_bps(P, c, dtype);
-                if (bps <= 0) continue;
+                const RowsCfg c = make_rows_cfg(G, sx, ty, tz, nt);
+                if (c.nchunks > 65535) continue;
                 const double blocks = (double)c.tiles * c.nchunks * (D == 4 ? G.n[2] : 1);
-                const double slots = (double)ctx->sm_count * bps;
+                const double slots = (double)sm_count * bps;
                 const double full = std::floor(blocks / slots), rest = blocks - full * slots;
-                const double per_sm = full * bps + std::ceil(rest / ctx->sm_count);
-                const double planes = (D >= 3 ? std::min(tz, ns) : 1) + 1.5;
+                const double per_sm = full * bps + std::ceil(rest / sm_count);
+                const double planes = (D >= 3 ? std::min(tz, ns) : 1) + prologue;
                 const double work = per_sm * (c.nt / 32.0) * planes;
-                const double latency = (full + (rest > 0 ? 1 : 0)) * 10.0 * planes;
-                scored.push_back({std::max(work, latency) + 0.1 * latency, c});
+                const double latency = (full + (rest > 0 ? 1 : 0)) * wave * planes;
+                scored.push_back({std::max(work, latency) + tail * latency, c});
             }
         }
     }
     std::sort(scored.begin(), scored.end(),
               [](const std::pair<double, RowsCfg>& a, const std::pair<double, RowsCfg>& b) { return a.first < b.first; });
     std::vector<RowsCfg> out;
-    for (size_t k = 0; k < scored.size() && k < 20; ++k) out.push_back(scored[k].second);
-    if (D == 2) {
+    for (const auto& c : scored) out.push_back(c.second);
+    return out;
+}
+
+// The shapes to time: the model's twenty best and, in 2-D, those of the plane kernel.
+std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtype) {
+    const GridDev& G = P.g;
+    const bool f64 = dtype == HJ_F64;
+    std::vector<RowsCfg> out = rows_ranked(P, dtype, ctx->sm_count, false);
+    if (out.size() > 20) out.resize(20);
+    if (G.ndim == 2) {
         // FP64 stages: 51^2 4.7 us with 7 x 6 nodes, 101^2 6.2 with 5 x 12, 201^2 9.2 with 16 x 9, 301^2 17.2
         // with 16 x 8, 511^2 44 (the row kernel 11.4, 13.8, 19.1, 50 from 101^2 on); FP32 takes 2.5 to 2.8 us
         // with either kernel up to 301^2
         static const int shapes[][2] = {{5, 8},  {5, 12}, {7, 4},  {7, 6},  {8, 5},   {8, 8},
                                         {12, 6}, {16, 8}, {16, 9}, {12, 12}, {16, 10}, {32, 8}};
-        for (const auto& sh : shapes) out.push_back(make_plane_cfg(G, std::min(sh[0], nx), std::min(sh[1], ny), f64));
+        for (const auto& sh : shapes) out.push_back(make_plane_cfg(G, std::min(sh[0], G.n[0]), std::min(sh[1], G.n[1]), f64));
     }
     return out;
 }

@@ -4,6 +4,8 @@
 
 #include <cstdint>
 #include <cuda_runtime.h>
+
+#include <vector>
 #include <nvtx3/nvToolsExt.h>
 
 namespace hj {
@@ -192,6 +194,10 @@ inline RowsCfg make_rows_cfg(const GridDev& G, int sx, int ty, int tz, int nt) {
     c.plane = 0;
     return c;
 }
+
+// The row kernel's launch shapes for this stage, the cheapest by a cost model first
+// (hj_api.cu; P finalized or not: its grid, dynamics and scheme count).
+std::vector<RowsCfg> rows_ranked(const StageParams& P, int dtype, int sm_count, bool quick);
 
 // The plane kernel's block: threads for the items of a tile (FP32: pairs of
 // interfaces), at most kPlaneThreads; and its shared memory.
