@@ -379,12 +379,20 @@ std::vector<RowsCfg> rows_ranked(const StageParams& P, int dtype, int sm_count, 
     return out;
 }
 
-// The shapes to time: the model's twenty best and, in 2-D, those of the plane kernel.
+// The shapes to time: the model's twenty best, the quick one's six best and, in
+// 2-D, those of the plane kernel.
 std::vector<RowsCfg> rows_candidates(hj_ctx* ctx, const StageParams& P, int dtype) {
     const GridDev& G = P.g;
     const bool f64 = dtype == HJ_F64;
     std::vector<RowsCfg> out = rows_ranked(P, dtype, ctx->sm_count, false);
     if (out.size() > 20) out.resize(20);
+    const std::vector<RowsCfg> quick = rows_ranked(P, dtype, ctx->sm_count, true);
+    for (size_t k = 0; k < quick.size() && k < 6; ++k) {
+        const RowsCfg& c = quick[k];
+        if (std::none_of(out.begin(), out.end(),
+                         [&c](const RowsCfg& o) { return o.sx == c.sx && o.ty == c.ty && o.tz == c.tz; }))
+            out.push_back(c);
+    }
     if (G.ndim == 2) {
         // FP64 stages: 51^2 4.7 us with 7 x 6 nodes, 101^2 6.2 with 5 x 12, 201^2 9.2 with 16 x 9, 301^2 17.2
         // with 16 x 8, 511^2 44 (the row kernel 11.4, 13.8, 19.1, 50 from 101^2 on); FP32 takes 2.5 to 2.8 us
@@ -459,15 +467,10 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
         cudaEvent_t e0, e1;
         HJ_CUDA(ctx, cudaEventCreate(&e0));
         HJ_CUDA(ctx, cudaEventCreate(&e1));
-        // Short launches are timed in rows of up to eight, as a step or a solve runs
-        // them: the event clock advances in steps of about two microseconds, and of
-        // a row only the first launch finds an empty chip. Where two blocks fit an
-        // SM, the next launch's blocks wait beside the running ones wherever there
-        // is room, some SMs get two of them and others none (103 x 47 x 44 FP64
-        // ENO3: a shape at 52 us a launch in pairs took 88 in a step; now 55 to 57).
-        const double per_us = dtype == HJ_F64 ? 4e3 : 4e4;  // nodes a microsecond, roughly
-        const int group = (int)std::min(8.0, std::max(1.0, std::ceil(600.0 * per_us / (double)G.total)));
-        const auto timed = [&](const RowsCfg& c, int reps, float* ms_min) -> cudaError_t {
+        // Short launches are timed in rows, as a step or a solve runs them: the event
+        // clock advances in steps of about two microseconds, and of a row only the
+        // first launch finds an empty chip.
+        const auto timed = [&](const RowsCfg& c, int group, int reps, float* ms_min) -> cudaError_t {
             cudaError_t e = cudaSuccess;
             for (int rep = 0; rep < reps && e == cudaSuccess; ++rep) {
                 cudaEventRecord(e0, ctx->stream);
@@ -476,26 +479,35 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
                 if (e == cudaSuccess) e = cudaEventSynchronize(e1);
                 float ms = 1e30f;
                 if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-                *ms_min = std::min(*ms_min, ms);
+                *ms_min = std::min(*ms_min, ms / group);
             }
             return e;
         };
-        // about a millisecond of launches first (an idle GPU's clocks rise meanwhile), every candidate once or twice,
-        // then the five best again: a pick by one disturbed group cost up to a third of a step
+        // A few launches first (an idle GPU's clocks rise meanwhile) tell how many make
+        // a row; every candidate once, then the five best again: a pick by one
+        // disturbed row cost up to a third of a step. (A first step of 101^2 FP64 takes
+        // 3.2 ms with it, of 61^3 FP64 14; with a millisecond of launches and rows of
+        // eight whatever they took, 4.5 and 21.)
         cudaError_t e = cudaSuccess;
-        const int warm = (int)std::min(64.0, std::max(1.0, 1000.0 * per_us / (double)G.total));
-        for (int k = 0; k < warm && e == cudaSuccess; ++k) e = rows_launch(ctx, T, cands[0], dtype);
+        float one = 1e30f;
+        e = rows_launch(ctx, T, cands[0], dtype);
+        if (e == cudaSuccess) e = timed(cands[0], 1, 1, &one);
+        if (e == cudaSuccess && one < 0.2f) e = timed(cands[0], 8, 3, &one);
+        const auto row = [one](double ms) { return (int)std::min(8.0, std::max(1.0, std::ceil(ms / one))); };
         std::vector<std::pair<float, size_t>> took;
         for (size_t i = 0; i < cands.size() && e == cudaSuccess; ++i) {
             e = rows_launch(ctx, T, cands[i], dtype);  // loads the kernel, fills the caches
             float ms = 1e30f;
-            if (e == cudaSuccess) e = timed(cands[i], group >= 4 ? 1 : 2, &ms);
+            const int in_row = row(one < 0.02f ? 0.04 : 0.1);
+            if (e == cudaSuccess) e = timed(cands[i], in_row, in_row == 1 ? 2 : 1, &ms);
             took.push_back({ms, i});
         }
         std::sort(took.begin(), took.end());
         if (took.size() > 5) took.resize(5);
-        for (auto& t : took)
-            if (e == cudaSuccess) e = timed(cands[t.second], 3, &t.first);
+        for (auto& t : took) {
+            t.first = 1e30f;
+            if (e == cudaSuccess) e = timed(cands[t.second], row(0.6), 3, &t.first);
+        }
         if (e != cudaSuccess) {
             cudaEventDestroy(e0);
             cudaEventDestroy(e1);

@@ -122,8 +122,9 @@ Pick g_pick[32];
 unsigned g_picks = 0;
 
 // Launch shape of the row kernel without timing, the same every time: the one that
-// the quick cost model ranks first (a fixed number of node threads and planes for
-// two blocks an SM left two waves where one would do: 101^3 FP64 ENO3 980 us a step, now 596; 31^4 FP32 93, now 65).
+// the quick cost model ranks first. A fixed number of node threads, and planes for
+// two blocks an SM, left two waves where one would do: 101^3 FP64 ENO3 980 us a
+// step, now 596; 31^4 FP32 WENO5 93, now 65.
 bool pick_rows(const StageParams& P, int dtype, int device, int sm_count, RowsCfg* c) {
     const GridDev& G = P.g;
     const int D = G.ndim;
