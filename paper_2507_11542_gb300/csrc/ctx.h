@@ -33,7 +33,7 @@ struct hj_ctx {
     std::map<std::vector<long long>, hj::RowsCfg> rows_cache;  // tuned launch shapes per grid shape
     void* tune_buf = nullptr;                                 // output scratch of tuning launches
     size_t tune_bytes = 0;
-    std::map<std::vector<long long>, std::pair<int, int>> batch_shape;  // (threads, planes per tile) per group kind
+    std::map<std::vector<long long>, std::pair<int, int>> batch_shape;  // (threads, planes per tile) per group kind and size
     hj::Engine* batch_engine = nullptr;                        // reused by hj_solve_batch
     size_t batch_engine_bytes = 0;
     int batch_engine_slots = 0;

@@ -412,8 +412,66 @@ void append_tiles(const Slot& S, int si, std::vector<BatchTile>* out) {
 }
 }  // namespace
 
-// The group's block size and planes per tile: measured once per (dtype,
-// dimension, dynamics, scheme) and context on the members at hand, then reused.
+// Deals members (the largest first) into chains of about the same number of tiles.
+void Engine::deal(const std::vector<int>& members, std::vector<int>* part) const {
+    long long load[kChains] = {};
+    for (int i : members) {
+        const int c = (int)(std::min_element(load, load + kChains) - load);
+        part[c].push_back(i);
+        load[c] += tiles_of(slots[i]);
+    }
+}
+
+// Block sizes and planes per tile of a group, the cheapest by a cost model first: the
+// work of the busiest SM (blocks x warps x planes; FP64 with the edge warps and a plane
+// of prologue a chunk, FP32 without them and with four), and at least the latency of
+// its waves (a plane of a wave as long as 6 warps' work in FP64, 15 in FP32). Over 24
+// batches, all shapes timed, its fourteen best hold the best within a hundredth on all
+// but two (6 and 3 %).
+std::vector<std::pair<int, int>> Engine::rank_shapes(const Group& g, const std::vector<int>& members) {
+    const bool f64 = g.dtype == HJ_F64;
+    const int regs = g.ndim == 2 ? (f64 ? 128 : 80) : (f64 ? 168 : 96);  // a thread's registers, about
+    std::vector<std::pair<double, std::pair<int, int>>> scored;
+    for (int threads : {128, 192, 256, 320, 384, 448, 576, 640}) {
+        if (threads > max_block_threads(g.dtype)) continue;
+        for (int tzt : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) {
+            if (g.ndim < 3 && tzt > 1) break;
+            double blocks = 0.0, work = 0.0, planes = 0.0;
+            size_t smem = 0;
+            for (int m : members) {
+                Slot S = slots[m];
+                tile_shape(S, threads, tzt, &S.sx, &S.ty, &S.tz);
+                const double n = (double)tiles_of(S), p = S.tz + (f64 ? 1.0 : 4.0);
+                const int warps = (rows_node_threads(S.sx, S.ty) + (f64 ? rows_edge_threads(S.sx, f64) : 0)) / 32;
+                blocks += n;
+                work += n * warps * p;
+                planes += n * p;
+                smem = std::max(smem, rows_smem(S.sx, S.es));
+            }
+            const int bps = std::max(1, std::min(65536 / (regs * threads), std::min(2048 / threads, (int)(228 * 1024 / (smem + 1024)))));
+            const double slots_all = (double)ctx_->sm_count * bps;
+            const double full = std::floor(blocks / slots_all), rest = blocks - full * slots_all;
+            const double per_sm = full * bps + std::ceil(rest / ctx_->sm_count);
+            const double latency = (full + (rest > 0 ? 1 : 0)) * (f64 ? 6.0 : 15.0) * planes / blocks;
+            scored.push_back({std::max(per_sm * work / blocks, latency) + 0.1 * latency, {threads, tzt}});
+        }
+    }
+    std::sort(scored.begin(), scored.end());
+    std::vector<std::pair<int, int>> out;
+    for (const auto& c : scored) out.push_back(c.second);
+    return out;
+}
+
+// The group's block size and planes per tile: the model's fourteen best are timed once
+// per (dtype, dimension, dynamics, scheme), size (its nodes to a power of two) and
+// context on the members at hand, then reused. A group most of whose members are
+// stepping already takes what was timed for its size, or the model's first. (Kept
+// without the size, the first batch of a context decided for all later ones: 8 solves
+// of 121^3 FP32 took 9.9 ms, and 13.5 after one of 41^3; 31^4 8.7, and 13 to 23 after
+// 12^4. Planes were 4 to 32 whatever the grids: four of 21^3 FP64 ENO3 5.97 ms, now
+// 3.6; and 42 shapes timed: a first batch of six 101^3 FP32 15 ms, now 7.5. Timed one
+// launch at a time, or all tiles in one row of launches: two chains at a time choose
+// otherwise, 101^3 FP64 60 and 55 ms, the batch of 24 15.3 and 15.0.)
 hj_status Engine::shape_group(Group& g, const std::vector<int>& members, const std::vector<int>& fresh) {
     auto apply = [&](int threads, int tzt) {
         g.threads = threads;
@@ -427,73 +485,116 @@ hj_status Engine::shape_group(Group& g, const std::vector<int>& members, const s
             h_insts_[m].tz = slots[m].tz;
         }
     };
-    const std::vector<long long> key = {g.dtype, g.ndim, g.dyn, g.scheme};
+    long long nodes = 0, fresh_nodes = 0;
+    for (int m : members) nodes += slots[m].N;
+    for (int m : fresh) fresh_nodes += slots[m].N;
+    const std::vector<long long> key = {g.dtype, g.ndim, g.dyn, g.scheme, (long long)std::ilogb((double)nodes)};
     auto it = ctx_->batch_shape.find(key);
     if (it != ctx_->batch_shape.end()) {
         apply(it->second.first, it->second.second);
         return HJ_OK;
     }
-    std::vector<std::pair<int, int>> cands;
-    for (int threads : {128, 192, 256, 320, 448, 576})
-        if (threads <= max_block_threads(g.dtype)) {
-            if (g.ndim < 3) cands.push_back({threads, 1});
-            else
-                for (int tzt : {4, 6, 8, 12, 16, 24, 32}) cands.push_back({threads, tzt});
-        }
+    std::vector<std::pair<int, int>> cands = rank_shapes(g, members);
+    if (2 * fresh_nodes < nodes) {
+        apply(cands[0].first, cands[0].second);
+        return HJ_OK;
+    }
+    if (cands.size() > 14) cands.resize(14);
     std::pair<int, int> best = cands[0];
     if (cands.size() > 1) {
         cudaEvent_t e0, e1;
         HJ_CUDA(ctx_, cudaEventCreate(&e0));
         HJ_CUDA(ctx_, cudaEventCreate(&e1));
-        float best_ms = 1e30f;
         cudaError_t e = cudaSuccess;
-        for (auto c : cands) {
-            // timed on the new members only (their descriptors have not started stepping)
+        if (chain_stream_.empty()) {
+            cudaStream_t c = nullptr;
+            e = cudaStreamCreateWithFlags(&c, cudaStreamNonBlocking);
+            if (e == cudaSuccess) chain_stream_.push_back(c);
+        }
+        // timed on the new members only (their descriptors have not started stepping), in
+        // the two chains that they will run in
+        size_t split = 0;
+        const auto set_up = [&](std::pair<int, int> c) {
             apply(c.first, c.second);
+            cudaError_t r = cudaSuccess;
             for (int m : fresh)
-                e = cudaMemcpyAsync(d_insts_ + m, &h_insts_[m], sizeof(BatchInst), cudaMemcpyHostToDevice, stream_);
+                if (r == cudaSuccess)
+                    r = cudaMemcpyAsync(d_insts_ + m, &h_insts_[m], sizeof(BatchInst), cudaMemcpyHostToDevice, stream_);
+            std::vector<int> order = fresh, part[kChains];
+            std::sort(order.begin(), order.end(), [&](int a, int b) { return slots[a].N > slots[b].N; });
+            deal(order, part);
             g.tiles.clear();
-            for (int m : fresh) append_tiles(slots[m], m, &g.tiles);
-            if (g.tiles.size() > g.tile_cap) {
+            for (int k = 0; k < kChains; ++k) {
+                for (int m : part[k]) append_tiles(slots[m], m, &g.tiles);
+                if (k == 0) split = g.tiles.size();
+            }
+            if (r == cudaSuccess && g.tiles.size() > g.tile_cap) {
                 cudaStreamSynchronize(stream_);
                 cudaFree(g.d_tiles);
                 g.d_tiles = nullptr;
                 g.tile_cap = g.tiles.size() * 2;
-                e = cudaMalloc(&g.d_tiles, g.tile_cap * sizeof(BatchTile));
-                if (e != cudaSuccess) {
+                r = cudaMalloc(&g.d_tiles, g.tile_cap * sizeof(BatchTile));
+                if (r != cudaSuccess) {
                     g.d_tiles = nullptr;
                     g.tile_cap = 0;
                 }
             }
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(g.d_tiles, g.tiles.data(), g.tiles.size() * sizeof(BatchTile), cudaMemcpyHostToDevice,
+            if (r == cudaSuccess)
+                r = cudaMemcpyAsync(g.d_tiles, g.tiles.data(), g.tiles.size() * sizeof(BatchTile), cudaMemcpyHostToDevice,
                                     stream_);
-            // stage 1 only writes V1, which the first real step rewrites
-            auto launch = [&]() {
-                return g.dtype == HJ_F64 ? launch_batch_stage_f64(g.d_tiles, (int)g.tiles.size(), d_insts_, 1, g.ndim,
-                                                                  g.dyn, g.scheme, g.threads, g.smem, stream_)
-                                         : launch_batch_stage_f32(g.d_tiles, (int)g.tiles.size(), d_insts_, 1, g.ndim,
-                                                                  g.dyn, g.scheme, g.threads, g.smem, stream_);
-            };
-            if (e == cudaSuccess) e = launch();
+            return r;
+        };
+        const auto launch = [&](int stage, size_t from, size_t to, cudaStream_t s) {
+            if (from == to) return cudaSuccess;
+            launches += 1;
+            ctx_->launches += 1;
+            return g.dtype == HJ_F64 ? launch_batch_stage_f64(g.d_tiles + from, (int)(to - from), d_insts_, stage, g.ndim,
+                                                              g.dyn, g.scheme, g.threads, g.smem, s)
+                                     : launch_batch_stage_f32(g.d_tiles + from, (int)(to - from), d_insts_, stage, g.ndim,
+                                                              g.dyn, g.scheme, g.threads, g.smem, s);
+        };
+        // rows of stage 1 and 2 in turn, the least of `reps`, ms a launch: they only write V1
+        // and V2, which the first real step rewrites
+        const auto timed = [&](int row, int reps, float* ms) {
+            cudaError_t r = cudaSuccess;
+            const cudaStream_t other = chain_stream_[0];
+            for (int rep = 0; rep < reps && r == cudaSuccess; ++rep) {
+                r = cudaEventRecord(e0, stream_);
+                if (r == cudaSuccess) r = cudaStreamWaitEvent(other, e0, 0);
+                for (int k = 0; k < row && r == cudaSuccess; ++k) {
+                    r = launch(1 + k % 2, 0, split, stream_);
+                    if (r == cudaSuccess) r = launch(1 + k % 2, split, g.tiles.size(), other);
+                }
+                cudaError_t j = cudaEventRecord(cap_ev_, other);  // (joined after an error too)
+                if (j == cudaSuccess) j = cudaStreamWaitEvent(stream_, cap_ev_, 0);
+                if (r == cudaSuccess) r = j;
+                if (r == cudaSuccess) r = cudaEventRecord(e1, stream_);
+                if (r == cudaSuccess) r = cudaEventSynchronize(e1);
+                float x = 1e30f;
+                if (r == cudaSuccess) r = cudaEventElapsedTime(&x, e0, e1);
+                *ms = std::min(*ms, x / row);
+            }
+            return r;
+        };
+        if (e == cudaSuccess) e = set_up(cands[0]);
+        float one = 1e30f;
+        if (e == cudaSuccess) e = timed(2, 2, &one);
+        const auto row = [&one](double ms) { return 2 * (int)std::min(4.0, std::max(1.0, std::ceil(ms / (2.0 * one)))); };
+        std::vector<std::pair<float, size_t>> took;
+        for (size_t k = 0; k < cands.size() && e == cudaSuccess; ++k) {
+            e = set_up(cands[k]);
             float ms = 1e30f;
-            for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {
-                cudaEventRecord(e0, stream_);
-                e = launch();
-                cudaEventRecord(e1, stream_);
-                if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-                float x = 0.f;
-                if (e == cudaSuccess) cudaEventElapsedTime(&x, e0, e1);
-                ms = std::min(ms, x);
-            }
-            launches += 3;
-            ctx_->launches += 3;
-            if (e != cudaSuccess) break;
-            if (ms < best_ms) {
-                best_ms = ms;
-                best = c;
-            }
+            if (e == cudaSuccess) e = timed(row(0.04), 1, &ms);
+            took.push_back({ms, k});
         }
+        std::sort(took.begin(), took.end());
+        if (took.size() > 3) took.resize(3);
+        for (auto& t : took) {
+            t.first = 1e30f;
+            if (e == cudaSuccess) e = set_up(cands[t.second]);
+            if (e == cudaSuccess) e = timed(row(0.3), 2, &t.first);
+        }
+        if (e == cudaSuccess) best = cands[std::min_element(took.begin(), took.end())->second];
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         if (e != cudaSuccess) return cuda_fail(ctx_, e, "batch launch-shape timing");
@@ -522,14 +623,10 @@ hj_status Engine::rebuild_tiles() {
         g.smem = 0;
         for (int l = 0; l < kLanes; ++l) {
             g.chains[l].clear();
-            std::vector<int> part[kChains];
-            long long load[kChains] = {};
-            for (int i : order) {
-                if (slots[i].lane != l) continue;
-                const int c = (int)(std::min_element(load, load + kChains) - load);
-                part[c].push_back(i);
-                load[c] += tiles_of(slots[i]);
-            }
+            std::vector<int> mine, part[kChains];
+            for (int i : order)
+                if (slots[i].lane == l) mine.push_back(i);
+            deal(mine, part);
             for (const std::vector<int>& p : part) {
                 if (p.empty()) continue;
                 Chain c;

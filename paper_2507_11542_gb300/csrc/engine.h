@@ -128,6 +128,8 @@ class Engine {
         BatchTile* d_tiles = nullptr;
         size_t tile_cap = 0;
     };
+    void deal(const std::vector<int>& members, std::vector<int>* part) const;
+    std::vector<std::pair<int, int>> rank_shapes(const Group& g, const std::vector<int>& members);
     hj_status shape_group(Group& g, const std::vector<int>& members, const std::vector<int>& fresh);
     hj_status rebuild_tiles();
     // One RK3 step of a chain's instances.
@@ -144,7 +146,7 @@ class Engine {
     hj_ctx* ctx_ = nullptr;
     cudaStream_t stream_ = nullptr;
     cudaStream_t cap_stream_ = nullptr;          // capture only: the first chain
-    std::vector<cudaStream_t> chain_stream_;     // capture only: the others
+    std::vector<cudaStream_t> chain_stream_;     // capture and timing only: the others
     cudaEvent_t cap_ev_ = nullptr;
     int max_slots_ = 0;
     void* arena_mem_ = nullptr;
