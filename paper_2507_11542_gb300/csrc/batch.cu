@@ -88,7 +88,7 @@ extern "C" hj_status hj_solve_batch(hj_ctx* ctx, int32_t n, const hj_problem* pr
             return fail(ctx, HJ_ENONFINITE, "problem %d: v0 holds NaN or Inf", idx);
         }
         while (eng->any_active()) {
-            if ((st = eng->run(kBlockSteps))) {
+            if ((st = eng->run(eng->block_steps(kBlockSteps)))) {
                 clear_engine(eng);
                 return st;
             }

@@ -726,6 +726,14 @@ void Engine::done_slots(std::vector<int>* out) const {
     }
 }
 
+int Engine::block_steps(int most) const {
+    if (!tiles_dirty_ && exec_[0]) return most;
+    long long left = 1;
+    for (const Slot& S : slots)
+        if (S.used && S.active) left = std::max(left, S.steps_total - S.k_host);
+    return (int)std::min<long long>(most, left);
+}
+
 hj_status Engine::run(int K) {
     NvtxRange range("batched steps");
     if (K <= 0 || !any_active()) return HJ_OK;

@@ -87,6 +87,10 @@ class Engine {
     hj_status activate(std::vector<int>* failed);
     // K RK3 steps of every active slot.
     hj_status run(int K);
+    // How many steps to run next, `most` at most: no more than are left where a graph
+    // has to be captured anyway (six steps of six 101^2 FP32 solves: 828 us of a
+    // call with sixteen captured in two chains, 450 so).
+    int block_steps(int most) const;
     bool any_active() const;
     // Active slots whose steps are all enqueued.
     void done_slots(std::vector<int>* out) const;

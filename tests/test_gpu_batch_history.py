@@ -37,3 +37,20 @@ def test_small_batch_first(dyn, small, large):
         batch(ctx, small, 1, 5)
         after = batch(ctx, large, 8, 20)
     assert after <= 1.2 * fresh
+
+
+def test_short_batch_launches_its_own_steps():
+    """Six steps of six solves: three stages and an advance a step and chain, two
+    chains, and two launches a problem at the start; not a block of sixteen steps."""
+    import torch
+    from paper_2507_11542_gb300 import solver
+    spec, V0 = W.double_integrator(61, 0.5)
+    m = lib_method(dynamics=1)
+    with solver.Context(0) as ctx:
+        ts = [5.5 * 0.8 / solver.step_bound(ctx, spec, m)]
+        V = to_dev(V0, "float32")
+        for _ in range(2):
+            outs, times, stats = solver.solve_batch(ctx, [spec] * 6, [m] * 6, [V] * 6, [ts] * 6)
+        torch.cuda.synchronize()
+    assert stats[0]["steps"] == 6
+    assert stats[0]["kernel_launches"] <= 6 * 4 * 2 + 6 * 2 + 6
