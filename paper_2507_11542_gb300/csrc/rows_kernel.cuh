@@ -87,9 +87,11 @@ template <typename T, int D, int DYN, int KIND>
 __device__ __forceinline__ T stage_value(const StageParams& P, const StageRun<T>& R, const T* par, const T* x, T c, T s,
                                          const T* S, const T* Q, const T* h, bool alpha_global, T center, T old, T& w) {
     T yd = lf_node<T, D, DYN>(P, par, x, c, s, S, Q, h, alpha_global);
-    // BRT min(0, .) as a clamp (+inf: none); FP64 on the bit pattern: positive values (and +NaN) become 0
+    // BRT min(0, .) as a clamp (+inf: none); FP64 on the high word: what is positive
+    // becomes 0, NaN of either sign (quiet: high word above infinity's) stays, since
+    // its sign depends on how it came about
     if constexpr (std::is_same<T, double>::value) {
-        if (R.brt0 && __double_as_longlong(yd) > 0) yd = 0.0;
+        if (R.brt0 && (unsigned)__double2hiint(yd) <= 0x7ff00000u) yd = 0.0;
     } else {
         yd = fminf(yd, R.brt0 ? 0.0f : INFINITY);
     }

@@ -53,3 +53,30 @@ def test_stage_keeps_infinite_and_largest_values(ctx, dyn, kernel, tile, mark, s
     np.testing.assert_array_equal(got[inf], want[inf])
     err = np.abs(got[~inf] - want[~inf])
     assert (err <= 3 * 2.0 ** -24 * (np.abs(old[~inf]) + np.abs(u[~inf]))).all()
+
+
+@pytest.mark.parametrize("dyn", [DI, NORM, AIR3D, DUBINS])
+@pytest.mark.parametrize("mark", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("scheme", [1, 2, 3, 5])
+@pytest.mark.parametrize("tile", [(0, 0, 0, 0), (3, 2, 0, 0)])
+def test_fp64_rule_leaves_nan(ctx, dyn, mark, scheme, tile):
+    """min(0, .) of a term that is NaN is NaN in FP64, as in the oracle: nodes beside
+    infinite or undefined ones do not look like nodes where nothing moves. Held on
+    the same nodes as the oracle's, but WENO5 of infinite data, whose weights the two
+    form differently (infinite or NaN), and ENO2/3 of NaN data, whose candidates the
+    kernel compares by their bits (NaN above everything, so that the other one is
+    taken; the oracle's comparison with NaN takes the right one)."""
+    from oracle import oracle as O
+    from paper_2507_11542_gb300 import solver
+    from helpers import oracle_method
+    n, periodic = GRIDS[dyn]
+    spec = W.GridSpec(n, (-1.0, -1.5, 0.0, 0.0)[:len(n)], (2.0, 1.0, 6.0, 2.0)[:len(n)], periodic)
+    V = np.asfortranarray(W.random_field(spec, 6))
+    V[np.random.default_rng(4).uniform(size=n) < 0.01] = mark
+    with np.errstate(all="ignore"):
+        want = O.term(spec, oracle_method(scheme=scheme, dynamics=dyn, brt=1), V)
+    got = to_host(solver.term(ctx, spec, lib_method(scheme=scheme, dynamics=dyn, brt=1, kernel=1, tile=tile), to_dev(V)), n)
+    assert np.isnan(want).any()
+    if (scheme == 5 and np.isinf(mark)) or (scheme in (2, 3) and np.isnan(mark)):
+        return
+    np.testing.assert_array_equal(np.isnan(got), np.isnan(want))
