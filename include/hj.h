@@ -199,7 +199,9 @@ hj_status hj_upwind(hj_ctx* ctx, const hj_grid* grid, const hj_method* method, i
 
 /* Lax-Friedrichs term ydot = Hg(x, (p- + p+)/2) + sum_d alpha_d (p+_d - p-_d)/2
  * (Sec. 4, Listing 5), clamped to min(0, ydot) when method->brt is
- * HJ_BRT_MIN0 (Sec. 6.1). Reads v, writes ydot (device). Asynchronous.
+ * HJ_BRT_MIN0 (Sec. 6.1). Reads v, writes ydot (device). Asynchronous. Where v is
+ * infinite or NaN the term is too or NaN; the clamp takes NaN for 0 in FP32 (and with
+ * kernel = NODE) and leaves it in FP64.
  * Errors: HJ_EINVAL, HJ_ECUDA. */
 hj_status hj_term(hj_ctx* ctx, const hj_grid* grid, const hj_method* method, int32_t dtype,
                   const void* v, void* ydot);
@@ -253,8 +255,8 @@ hj_status hj_solve(hj_ctx* ctx, const hj_problem* problem, void* out_slices, int
  * solved one by one with hj_solve. Every problem is validated before any work;
  * results equal those of hj_solve on each problem alone (same arithmetic per
  * node). elapsed_ms and kernel_launches in stats are those of the whole call.
- * The first batch with a new (element type, dimension, dynamics, scheme) group times a
- * few launch shapes. Synchronises the stream.
+ * The first batch with a new (element type, dimension, dynamics, scheme) group, or with
+ * twice or half the nodes, times a few launch shapes. Synchronises the stream.
  * Errors: HJ_EINVAL (names the problem index), HJ_ENOMEM, HJ_ENONFINITE, HJ_ECUDA. */
 hj_status hj_solve_batch(hj_ctx* ctx, int32_t n, const hj_problem* problems, void* const* out_slices,
                          const int32_t* out_on_device, double* const* out_times, hj_stats* stats);

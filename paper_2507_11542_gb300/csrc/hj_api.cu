@@ -421,8 +421,8 @@ hj_status rows_config(hj_ctx* ctx, const StageParams& P, int dtype, const int32_
             *out = hit->second;
             return HJ_OK;
         }
-        // which shapes fit is a matter of nodes a block (hj.h): n0 nodes by ty
-        // rows, occ 2 for FP32 blocks of up to 544 threads of one node each
+        // which shapes fit is a rule of the interface (hj.h), kept although the kernel no
+        // longer needs it: n0 nodes by ty rows, occ 2 for FP32 blocks of up to 544 nodes
         const int tz = tile[1] > 0 ? tile[1] : 1, merged = tile[3] & 1, most = rows_max_nodes(dtype == HJ_F64);
         const long long nx = G.n[0], want = tile[0];
         bool fits = want <= G.n[1] && want <= nx && (nx + 1 - merged) * want <= most;

@@ -93,9 +93,8 @@ struct StageParams {
     double alpha_g[kMaxDim];
     int alpha_box;                // dissipation alpha_d = max |dHg/dp_d| over the node's box of gradients
     // FP32 copies of the scalars above, so that FP32 kernels do no FP64 arithmetic
-    float lo_f[kMaxDim], dx_f[kMaxDim], inv_dx_f[kMaxDim], half_inv_dx_f[kMaxDim], half_inv_dx6_f[kMaxDim];
+    float lo_f[kMaxDim], dx_f[kMaxDim], half_inv_dx_f[kMaxDim], half_inv_dx6_f[kMaxDim];
     float alpha_g_f[kMaxDim];
-    float weno_floor_f[kMaxDim];
     float params_f[8];
     float dt_f, cv_f, cu_f;
     int has_vn;            // the stage reads Vn (cv != 0 or minv_after)
@@ -110,13 +109,11 @@ inline StageParams finalize(StageParams p) {
     for (int d = 0; d < kMaxDim; ++d) {
         p.lo_f[d] = (float)p.g.lo[d];
         p.dx_f[d] = (float)p.g.dx[d];
-        p.inv_dx_f[d] = (float)p.g.inv_dx[d];
         p.half_inv_dx[d] = 0.5 * p.g.inv_dx[d];
         p.half_inv_dx6[d] = p.half_inv_dx[d] / 6.0;
         p.half_inv_dx6_f[d] = (float)p.half_inv_dx6[d];
         p.half_inv_dx_f[d] = (float)p.half_inv_dx[d];
         p.alpha_g_f[d] = (float)p.alpha_g[d];
-        p.weno_floor_f[d] = (float)p.weno_floor[d];
         p.weno_floor12[d] = 12.0 * p.weno_floor[d];
     }
     for (int k = 0; k < 8; ++k) p.params_f[k] = (float)p.params[k];

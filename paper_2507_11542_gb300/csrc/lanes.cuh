@@ -2,8 +2,10 @@
 // thread of the row kernel works on. FP32 pairs live in one 64-bit register
 // pair and use the packed instructions of this GPU (add, mul and fma on two
 // floats at once: the same rate per operation as the scalar ones, half the
-// instructions to issue); FP64 pairs are two doubles. Every operation rounds
-// once, like the scalar one; none is left for the compiler to contract.
+// instructions to issue); FP64 pairs are two doubles. FP64 operations round once
+// each; of the packed ones only fma2 is a single rounding for certain: a product
+// whose only use is a sum may be fused with it, so that code which has to round
+// alike in every inlined copy leaves none (weno_iface2).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -93,8 +93,8 @@ __device__ __forceinline__ void weno_iface2(F2 e1, F2 e2, F2 e3, F2 e4, F2 e5, F
 
 // 1/x for a positive normal double: the hardware estimate refined by two
 // Newton-Raphson steps r <- r + r (1 - x r) (each squares the relative error).
-// The interface no longer needs it (its reciprocals are integer); it stays as
-// the library's FP64 reciprocal, held against 1/x by its test.
+// Nothing in the library calls it since the interface's reciprocals are integer;
+// its test (test_gpu_rcp.py) does.
 __device__ __forceinline__ double rcp_newton(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));

@@ -5,9 +5,9 @@
 // in which the four schedulers issue 64 to 80 others. An interface's weights
 // are the bulk of its arithmetic, and they are products, sums of positive
 // numbers and two reciprocals: with 63-bit integer mantissas and integer
-// exponents they need no FP64 instruction, and keep more bits than FP64 does
-// (every product is good to 2^-58 or better, so the weights' error is
-// their final rounding to FP64). Measured on a sweep over columns in L2, SM
+// exponents they need no FP64 instruction. Products are good to 2^-58, smoothness
+// sums to 2^-54 and the weights to a few units of 2^-53 (2.3 at most against exact
+// rationals; 2^-51 is what the sums' error allows). Measured on a sweep over columns in L2, SM
 // cycles per warp interface: from six values 1272 with FP64 weights and 460 with
 // these, along a line (Weno5Line) 1009 and 298.
 //
