@@ -10,8 +10,8 @@
 // through shared memory, and each node is updated by a thread of its own: 6.2 us
 // (5 x 12 nodes a block, two blocks an SM), 44 us instead of 50 on 511^2; a whole
 // solve of 101^2 then took 2592 us, with the smoothness sums in integers 2438, and
-// with indices and cells ready before the wait for the kernel in front 2275. FP32,
-// whose stage is launch latency up to 301^2 (2.5 to 2.8 us with either kernel),
+// with indices and cells ready before the wait for the kernel in front 2275, with
+// the next kernel let in only after that wait 1800. FP32, whose stage is launch latency up to 301^2 (2.5 to 2.8 us with either kernel),
 // keeps the row kernel where that is faster: the launch-shape tuner times both.
 // Both evaluate an interface and a node with the same functions, so that the
 // results are the same bits.

@@ -132,7 +132,12 @@ bool pick_rows(const StageParams& P, int dtype, int device, int sm_count, RowsCf
     for (int d = 0; d < D; ++d)
         if (G.n[d] < 4) return false;
     if (G.n[0] + 1 > rows_max_nodes(dtype == HJ_F64)) return false;
-    if (D == 2 && dtype == HJ_F64) {  // 101^2: 6.2 us a stage, the row kernel 11.4; 511^2: 44 and 50
+    if (D == 2 && dtype == HJ_F64) {
+        // The plane kernel at every size (WENO5, a stage: 101^2 6.2 us, the row kernel 11.4; 511^2: 44 and 50). Tiles of
+        // 5x12 while they leave the chip idle, 16x8 (a smaller halo) above. WENO5, us per step, 5x12 and 16x8: 51^2 12.7
+        // and 14.7, 101^2 15.0 and 15.1, 122^2 15.5 and 15.2, 131^2 15.4 and 16.9, 151^2 27.2 and 20.9, 201^2 27.9 and
+        // 27.8, 301^2 57.2 and 47.0, 511^2 136 and 120; ENO2: 101^2 10.2 and 11.8, 151^2 14.6 and 14.9, 201^2 19.4 and
+        // 18.6. Between 101^2 and 141^2 the two are within a tenth of each other; the line lies in the middle of that.
         *c = G.total < 15000 ? make_plane_cfg(G, std::min(5, G.n[0]), std::min(12, G.n[1]), 1)
                              : make_plane_cfg(G, std::min(16, G.n[0]), std::min(8, G.n[1]), 1);
         return true;
